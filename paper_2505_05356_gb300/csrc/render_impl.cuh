@@ -48,6 +48,21 @@ constexpr int rec_stride() {
   return sizeof(Real) == 4 ? RecStrideF<F>::value : RecStrideD<F>::value;
 }
 
+// The word after the features, 1/o and d is padding in every record; a staged
+// record carries its place in the tile's list there (as bits), so the walk
+// gets it with the record instead of from an array of its own.
+template <int F>
+constexpr int kIdxWord = 8 + 2 * F + 1;
+static_assert(kIdxWord<1> < RecStrideF<1>::value && kIdxWord<2> < RecStrideF<2>::value &&
+              kIdxWord<3> < RecStrideF<3>::value && kIdxWord<4> < RecStrideF<4>::value &&
+              kIdxWord<1> < RecStrideD<1>::value && kIdxWord<2> < RecStrideD<2>::value &&
+              kIdxWord<3> < RecStrideD<3>::value && kIdxWord<4> < RecStrideD<4>::value,
+              "a record has a padding word");
+__device__ __forceinline__ void put_index(float* w, uint32_t i) { *w = __uint_as_float(i); }
+__device__ __forceinline__ void put_index(double* w, uint32_t i) { *w = __longlong_as_double(i); }
+__device__ __forceinline__ uint32_t get_index(float w) { return __float_as_uint(w); }
+__device__ __forceinline__ uint32_t get_index(double w) { return (uint32_t)__double_as_longlong(w); }
+
 // one rounding per operation, so forward and backward evaluate alpha with
 // bit-identical results (the backward replays the forward's decisions)
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
@@ -96,6 +111,24 @@ struct Fold<LEN, 0> {
   template <typename Real>
   static __device__ __forceinline__ void run(Real*, int) {}
 };
+
+// The backward's sums over a warp, single precision: instead of a shuffle
+// butterfly per record (12 shuffles, 12 adds and 24 selects for nine values),
+// the lanes write their values to rows of shared memory (one row of 32 lanes
+// per value) and, once kRowRecords<GS> records fill the rows, lane i adds up
+// row i and owns that sum: 9 stores per record and 8 loads + 17 packed adds
+// per three records instead of some 50 instructions per record of a kernel
+// that is bound by instruction issue.  With the list place in the record and
+// a constant CTA size (fewer registers) the backward of 16 frames of 300k
+// Gaussians went from 1.22 to 1.00 ms (step 2.397 -> 2.172 ms).  Every lane's
+// row takes its eight 16-byte chunks starting from its own, so a quarter warp
+// reads eight distinct chunks and no bank twice.
+template <int GS>
+constexpr int kRowRecords = 32 / GS;  // records whose values fit 32 rows
+template <typename Real, int GS>
+constexpr int row_floats() {  // per warp; the double instantiation folds by shuffles
+  return sizeof(Real) == 4 ? kRowRecords<GS> * GS * 32 : 0;
+}
 
 // value index whose warp total lane `lane` ends with after Fold<GS, 16>;
 // -1 for lanes that end with padding only
@@ -231,12 +264,13 @@ __device__ __forceinline__ int block_compact(bool keep, int* s_cnt, int& pos) {
   return total;
 }
 
-// number of entries of the increasing array a[0..n) below x
-__device__ __forceinline__ int count_below(const uint32_t* a, int n, uint32_t x) {
+// number of the staged records rec[0..n) (stride RS) whose list place is below x
+template <int F, int RS, typename Real>
+__device__ __forceinline__ int count_below(const Real* rec, int n, uint32_t x) {
   int lo = 0, hi = n;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
-    if (a[mid] < x)
+    if (get_index(rec[mid * RS + kIdxWord<F>]) < x)
       lo = mid + 1;
     else
       hi = mid;
@@ -297,11 +331,35 @@ __device__ __forceinline__ F2 fma2_rn(F2 a, F2 b, F2 c) {
   return r;
 }
 
-// log2_oG of the PPT pixels of one column: pairs of pixels in packed FP32x2
+__device__ __forceinline__ F2 add2_rn(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+
+// this lane's row of 32 values (kRowRecords): 16-byte chunks from the lane's own on
+__device__ __forceinline__ float row_sum(const float* row, int lane) {
+  const ulonglong2* p = reinterpret_cast<const ulonglong2*>(row);
+  ulonglong2 v = p[lane & 7];
+  F2 a{v.x}, b{v.y};
+#pragma unroll
+  for (int q = 1; q < 8; ++q) {
+    v = p[(lane + q) & 7];
+    a = add2_rn(a, F2{v.x});
+    b = add2_rn(b, F2{v.y});
+  }
+  float lo, hi;
+  unpack2(add2_rn(a, b), lo, hi);
+  return lo + hi;
+}
+// (never called: the double instantiation folds by shuffles)
+__device__ __forceinline__ double row_sum(const double*, int) { return 0.0; }
+
+// log2_oG and dy of the PPT pixels of one column: pairs of pixels in packed FP32x2
 // (the same roundings as log2_oG); the double instantiation stays scalar
 template <int PPT>
 __device__ __forceinline__ void log2_oG_column(const float* r, const Column<float>& c,
-                                               const float* fpy, float* lg) {
+                                               const float* fpy, float* lg, float* dyv) {
   if constexpr (PPT % 2 == 0) {
     const F2 r1 = pack2(r[1], r[1]), r4 = pack2(r[4], r[4]);
     const F2 cb = pack2(c.cb_dx, c.cb_dx), alo = pack2(c.a_lo, c.a_lo);
@@ -309,17 +367,24 @@ __device__ __forceinline__ void log2_oG_column(const float* r, const Column<floa
     for (int h = 0; h < PPT / 2; ++h) {
       const F2 dy = sub2_rn(r1, pack2(fpy[2 * h], fpy[2 * h + 1]));
       unpack2(fma2_rn(fma2_rn(r4, dy, cb), dy, alo), lg[2 * h], lg[2 * h + 1]);
+      unpack2(dy, dyv[2 * h], dyv[2 * h + 1]);
     }
   } else {
 #pragma unroll
-    for (int k = 0; k < PPT; ++k) lg[k] = log2_oG(r, c, sub_rn(r[1], fpy[k]));
+    for (int k = 0; k < PPT; ++k) {
+      dyv[k] = sub_rn(r[1], fpy[k]);
+      lg[k] = log2_oG(r, c, dyv[k]);
+    }
   }
 }
 template <int PPT>
 __device__ __forceinline__ void log2_oG_column(const double* r, const Column<double>& c,
-                                               const double* fpy, double* lg) {
+                                               const double* fpy, double* lg, double* dyv) {
 #pragma unroll
-  for (int k = 0; k < PPT; ++k) lg[k] = log2_oG(r, c, sub_rn(r[1], fpy[k]));
+  for (int k = 0; k < PPT; ++k) {
+    dyv[k] = sub_rn(r[1], fpy[k]);
+    lg[k] = log2_oG(r, c, dyv[k]);
+  }
 }
 
 // Resident CTAs per SM the compiler is asked to fit (register budget).  Only
@@ -328,12 +393,19 @@ __device__ __forceinline__ void log2_oG_column(const double* r, const Column<dou
 // threads (32x32 tile, WIDE) 3 of either (<= 85).
 template <int PPT, bool BWD, bool WIDE>
 struct kMinBlocks {
-  static constexpr int value = WIDE ? 3 : (PPT == 4 ? (BWD ? 6 : 7) : 0);
+  static constexpr int value =
+      WIDE ? 3 : (PPT == 4 ? (BWD ? 6 : 7) : (BWD ? (PPT == 2 ? 3 : 2) : 0));
 };
 template <int PPT, bool WIDE>
 struct kMaxThreads {
   static constexpr int value = (WIDE ? 1024 : 512) / PPT;
 };
+// threads of the CTA: a 32x32 part always has all of them, so that offsets in
+// its shared memory are constants instead of registers
+template <int PPT, bool WIDE>
+__device__ __forceinline__ int cta_threads() {
+  return WIDE ? kMaxThreads<PPT, WIDE>::value : (int)blockDim.x;
+}
 
 template <typename Real, int F, int PPT, bool DEPTH, bool COUNT>
 __device__ __forceinline__ void render_tile_fwd(
@@ -341,8 +413,7 @@ __device__ __forceinline__ void render_tile_fwd(
     const uint2* __restrict__ ranges, const uint32_t* __restrict__ values,
     const Real* __restrict__ rec, const Real* __restrict__ bg,
     Real* __restrict__ out, Real* __restrict__ tfinal,
-    uint32_t* __restrict__ nlast, Real* s_rec, Real* s_stage, uint32_t* s_idx,
-    int* s_cnt, unsigned* s_mask, Header* __restrict__ hdr) {
+    uint32_t* __restrict__ nlast, Real* s_rec, Real* s_stage, int* s_cnt, unsigned* s_mask, Header* __restrict__ hdr) {
   constexpr int NF = 2 * F + 1;
   constexpr int RS = rec_stride<Real, F>();
   constexpr unsigned ALL = (1u << PPT) - 1u;
@@ -405,7 +476,7 @@ __device__ __forceinline__ void render_tile_fwd(
       float4* dst = reinterpret_cast<float4*>(s_rec + pos * RS);
 #pragma unroll
       for (int k = 0; k < V4; ++k) dst[k] = stg[k];
-      s_idx[pos] = i;
+      put_index(s_rec + pos * RS + kIdxWord<F>, i);
     }
     __syncthreads();
     // records that can reach alpha_min at a pixel centre of this warp's block
@@ -435,11 +506,11 @@ __device__ __forceinline__ void render_tile_fwd(
         const Column<Real> col = column_of(r, fpx);
         // the exponents of all PPT pixels first (independent chains), then
         // each pixel's decisions
-        Real lg[PPT], oG[PPT];
-        log2_oG_column<PPT>(r, col, fpy, lg);
+        Real lg[PPT], oG[PPT], dyv[PPT];
+        log2_oG_column<PPT>(r, col, fpy, lg, dyv);
 #pragma unroll
         for (int k = 0; k < PPT; ++k) oG[k] = ex2_approx(lg[k]);
-        const uint32_t jn = s_idx[j] + 1;  // list entries up to this one
+        const uint32_t jn = get_index(r[kIdxWord<F>]) + 1;  // list entries up to this one
 #pragma unroll
         for (int k = 0; k < PPT; ++k) {
           if (done & (1u << k)) continue;
@@ -515,7 +586,6 @@ __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real* s_rec = reinterpret_cast<Real*>(smem_raw);
   Real* s_stage = s_rec + (size_t)blockDim.x * RS;
-  uint32_t* s_idx = reinterpret_cast<uint32_t*>(s_stage + (size_t)blockDim.x * RS);
   __shared__ int s_cnt[32];
   __shared__ unsigned s_mask[kMaskWords * kMaskWords];  // [warp][word]
   const uint32_t items = (uint32_t)rg.B * rg.NT * rg.S;
@@ -523,7 +593,7 @@ __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
     const uint32_t item = blockIdx.y * rg.NT * rg.S + blockIdx.x;
     render_tile_fwd<Real, F, PPT, DEPTH, COUNT>(tile_of(item, rg), rg, tab, ranges,
                                          values, rec, bg, out, tfinal, nlast, s_rec, s_stage,
-                                         s_idx, s_cnt, s_mask, hdr);
+                                         s_cnt, s_mask, hdr);
     return;
   }
   __shared__ uint32_t s_item;
@@ -535,14 +605,14 @@ __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
     if (item >= items) break;
     render_tile_fwd<Real, F, PPT, DEPTH, COUNT>(tile_of(item, rg), rg, tab, ranges,
                                          values, rec, bg, out, tfinal, nlast, s_rec, s_stage,
-                                         s_idx, s_cnt, s_mask, hdr);
+                                         s_cnt, s_mask, hdr);
   }
 }
 
 // ---------------------------------------------------------------------------
 // backward
 // ---------------------------------------------------------------------------
-template <typename Real, int F, int PPT, bool DEPTH>
+template <typename Real, int F, int PPT, bool DEPTH, bool WIDE>
 __device__ __forceinline__ void render_tile_bwd(
     const TileCtx& tc, const RenderGeom& rg, const TableT<Real>* __restrict__ tab,
     const uint2* __restrict__ ranges, const uint32_t* __restrict__ values,
@@ -550,11 +620,11 @@ __device__ __forceinline__ void render_tile_bwd(
     const Real* __restrict__ dout, const Real* __restrict__ tfinal,
     const uint32_t* __restrict__ nlast, Real* __restrict__ g2d, int g2d_stride,
     Real* __restrict__ dbg, Real* s_rec, Real* s_grad, uint32_t* s_id,
-    Real* s_red, uint32_t* s_idx, int* s_cnt, Real* s_stage, unsigned* s_mask) {
+    Real* s_red, int* s_cnt, Real* s_stage, unsigned* s_mask) {
   constexpr int NF = 2 * F + 1;
   constexpr int GS = 6 + NF + (DEPTH ? 1 : 0);
   constexpr int RS = rec_stride<Real, F>();
-  const int nthr = blockDim.x, tid = threadIdx.x;
+  const int nthr = cta_threads<PPT, WIDE>(), tid = threadIdx.x;
   const int lane = tid & 31, wid = tid >> 5, nwarps = nthr >> 5;
   const ThreadPix tp = thread_pixels<PPT>(tid, rg.CW);
   const int lx = tp.lx, ly0 = tp.ly0;
@@ -629,12 +699,10 @@ __device__ __forceinline__ void render_tile_bwd(
     }
   }
   // longest list any pixel of the tile needs
-  int maxn = thread_n;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) maxn = max(maxn, __shfl_xor_sync(0xffffffffu, maxn, o));
-  if (lane == 0) reinterpret_cast<int*>(s_red)[wid] = maxn;
+  const int warp_n = __reduce_max_sync(0xffffffffu, thread_n);  // ... any of the warp's
+  if (lane == 0) reinterpret_cast<int*>(s_red)[wid] = warp_n;
   __syncthreads();
-  maxn = 0;
+  int maxn = 0;
   for (int w = 0; w < nwarps; ++w) maxn = max(maxn, reinterpret_cast<int*>(s_red)[w]);
   __syncthreads();
 
@@ -650,7 +718,12 @@ __device__ __forceinline__ void render_tile_bwd(
     A[k] = 0;
     BD[k] = 0;
   }
-  const int red_slot = butterfly_slot<GS>(lane);
+  // single precision: rows of per-lane values in shared memory (the stage
+  // slots' space, free between the staging barriers); lane i sums row i, value
+  // i % GS of the rows' record i / GS.  Double: shuffle butterfly.
+  constexpr bool ROWS = sizeof(Real) == 4;
+  const int red_slot = ROWS ? 0 : butterfly_slot<GS>(lane);
+  Real* const rows = s_stage + wid * row_floats<Real, GS>() + lane;  // this lane's column
   const Real ln2 = Real(kLn2);
   Real* gbase = g2d + (size_t)tc.b * rg.N * g2d_stride;
 
@@ -683,23 +756,14 @@ __device__ __forceinline__ void render_tile_bwd(
       float4* dst = reinterpret_cast<float4*>(s_rec + pos * RS);
 #pragma unroll
       for (int k = 0; k < V4; ++k) dst[k] = stg[k];
+      put_index(s_rec + pos * RS + kIdxWord<F>, (uint32_t)(lo + tid));
       s_id[pos] = g;
-      s_idx[pos] = (uint32_t)(lo + tid);
     }
     for (int k = tid; k < nk * GS; k += nthr) s_grad[k] = Real(0);
     __syncthreads();
-    // staged entries [0, my_hi[k]) precede pixel k's last composited one;
-    // warps whose pixels all stop before the batch skip it
-    int my_hi[PPT];
-    int thread_hi = 0;
-#pragma unroll
-    for (int k = 0; k < PPT; ++k) {
-      my_hi[k] = count_below(s_idx, nk, (uint32_t)nl[k]);
-      thread_hi = max(thread_hi, my_hi[k]);
-    }
-    int warp_hi = thread_hi;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) warp_hi = max(warp_hi, __shfl_xor_sync(0xffffffffu, warp_hi, o));
+    // staged entries [0, warp_hi) precede the last one composited by any of the
+    // warp's pixels; warps whose pixels all stop before the batch skip it
+    const int warp_hi = count_below<F, RS>(s_rec, nk, (uint32_t)warp_n);
     // records below warp_hi that can reach alpha_min in this warp's block (the
     // forward's warp test, so the same records): bit j of word q is 32 q + j
     const int nq = (warp_hi + 31) >> 5;
@@ -711,6 +775,16 @@ __device__ __forceinline__ void render_tile_bwd(
       if (lane == 0) s_mask[wid * kMaskWords + q] = m;
     }
     __syncwarp();
+    int filled = 0, red_dst = 0;  // rows in use; where this lane's sum goes
+    auto add_rows = [&]() {
+      __syncwarp();
+      if (lane < filled) {
+        const Real t = row_sum(rows + lane * 31, lane);
+        if (t != Real(0)) atomicAdd(&s_grad[red_dst], t);
+      }
+      __syncwarp();
+      filled = 0;
+    };
     for (int q = nq - 1; q >= 0; --q) {
      unsigned m = s_mask[wid * kMaskWords + q];
      while (m) {
@@ -722,19 +796,20 @@ __device__ __forceinline__ void render_tile_bwd(
 #pragma unroll
       for (int q = 0; q < GS; ++q) c[q] = 0;
       bool has = false;
-      if (j < thread_hi) {
+      const int place = (int)get_index(r[kIdxWord<F>]);
+      {
         const Column<Real> col = column_of(r, fpx);
         // moments over this thread's pixels (same column) of dL/dpower:
         // S0 = sum d, S1 = sum d dy, S2 = sum d dy^2 (S0 is also the sum of
         // dL/dalpha o G: where alpha is not clamped, d = dL/dalpha alpha and
         // alpha = o G)
         Real S0 = 0, S1 = 0, S2 = 0;
-        Real lgv[PPT];  // exponents of all PPT pixels first (packed pairs)
-        log2_oG_column<PPT>(r, col, fpy, lgv);
+        Real lgv[PPT], dyv[PPT];  // exponents of all PPT pixels first (packed pairs)
+        log2_oG_column<PPT>(r, col, fpy, lgv, dyv);
 #pragma unroll
         for (int k = 0; k < PPT; ++k) {
-          if (j >= my_hi[k]) continue;
-          const Real dy = sub_rn(r[1], fpy[k]);
+          if (place >= nl[k]) continue;  // after the pixel's last composited one
+          const Real dy = dyv[k];
           const Real lg = lgv[k];
           const Real oG = ex2_approx(lg);
           const Real alpha = oG < amax ? oG : amax;
@@ -783,11 +858,21 @@ __device__ __forceinline__ void render_tile_bwd(
         }
       }
       if (__any_sync(0xffffffffu, has)) {
-        Fold<GS, 16>::run(c, lane);
-        if (red_slot >= 0 && c[0] != Real(0)) atomicAdd(&s_grad[j * GS + red_slot], c[0]);
+        if constexpr (ROWS) {
+          Real* row = rows + filled * 32;
+#pragma unroll
+          for (int q = 0; q < GS; ++q) row[q * 32] = c[q];
+          if ((unsigned)(lane - filled) < (unsigned)GS) red_dst = j * GS + lane - filled;
+          filled += GS;
+          if (filled == kRowRecords<GS> * GS) add_rows();
+        } else {
+          Fold<GS, 16>::run(c, lane);
+          if (red_slot >= 0 && c[0] != Real(0)) atomicAdd(&s_grad[j * GS + red_slot], c[0]);
+        }
       }
      }
     }
+    if (filled > 0) add_rows();
     __syncthreads();
     // per record: the 2D gradient from the CTA's sums (alpha = 2^(log2 o +
     // ln2-scaled quadratic), d alpha / d o = alpha / o), one global atomic per
@@ -829,21 +914,20 @@ __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
   constexpr int GS = 6 + NF + (DEPTH ? 1 : 0);
   constexpr int RS = rec_stride<Real, F>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int nthr = blockDim.x;
+  const int nthr = cta_threads<PPT, WIDE>();
   Real* s_rec = reinterpret_cast<Real*>(smem_raw);
   Real* s_grad = s_rec + (size_t)nthr * RS;
   Real* s_red = s_grad + (size_t)nthr * GS;
   uint32_t* s_id = reinterpret_cast<uint32_t*>(s_red + 32);
-  uint32_t* s_idx = s_id + nthr;
-  Real* s_stage = reinterpret_cast<Real*>(s_idx + nthr);
+  Real* s_stage = reinterpret_cast<Real*>(s_id + nthr);
   __shared__ int s_cnt[32];
   __shared__ unsigned s_mask[kMaskWords * kMaskWords];  // [warp][word]
   const uint32_t items = (uint32_t)rg.B * rg.NT * rg.S;
   if (!persistent) {
     const uint32_t item = blockIdx.y * rg.NT * rg.S + blockIdx.x;
-    render_tile_bwd<Real, F, PPT, DEPTH>(tile_of(item, rg), rg, tab, ranges,
+    render_tile_bwd<Real, F, PPT, DEPTH, WIDE>(tile_of(item, rg), rg, tab, ranges,
                                   values, rec, bg, dout, tfinal, nlast, g2d,
-                                  g2d_stride, dbg, s_rec, s_grad, s_id, s_red, s_idx, s_cnt,
+                                  g2d_stride, dbg, s_rec, s_grad, s_id, s_red, s_cnt,
                                   s_stage, s_mask);
     return;
   }
@@ -854,9 +938,9 @@ __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
     const uint32_t item = s_item;
     __syncthreads();
     if (item >= items) break;
-    render_tile_bwd<Real, F, PPT, DEPTH>(tile_of(item, rg), rg, tab, ranges,
+    render_tile_bwd<Real, F, PPT, DEPTH, WIDE>(tile_of(item, rg), rg, tab, ranges,
                                   values, rec, bg, dout, tfinal, nlast, g2d,
-                                  g2d_stride, dbg, s_rec, s_grad, s_id, s_red, s_idx, s_cnt,
+                                  g2d_stride, dbg, s_rec, s_grad, s_id, s_red, s_cnt,
                                   s_stage, s_mask);
   }
 }
@@ -886,7 +970,7 @@ void fwd_launch(const Layout& L, const Real* bg, Real* out, unsigned char* ws,
   constexpr int RS = rec_stride<Real, F>();
   const RenderGeom rg = geom_of(L);
   const int threads = rg.CW * rg.CH / PPT;
-  const size_t smem = (size_t)threads * (2 * RS * sizeof(Real) + sizeof(uint32_t));
+  const size_t smem = (size_t)threads * 2 * RS * sizeof(Real);
   auto kernel = render_fwd_kernel<Real, F, PPT, DEPTH, COUNT, WIDE>;
   static PerDeviceOnce attr;
   attr.run([&] {
@@ -908,6 +992,10 @@ void fwd_launch(const Layout& L, const Real* bg, Real* out, unsigned char* ws,
   count_launches(1);
 }
 
+// dynamic shared memory of a backward CTA, at most (512 threads and 16 values:
+// four frequencies with the depth channel)
+constexpr int kMaxBwdSmem = 160 * 1024;
+
 template <typename Real, int F, int PPT, bool DEPTH, bool WIDE>
 void bwd_launch(const Layout& L, const Real* bg, const Real* dout, Real* dbg,
                 unsigned char* ws, cudaStream_t st) {
@@ -916,13 +1004,16 @@ void bwd_launch(const Layout& L, const Real* bg, const Real* dout, Real* dbg,
   constexpr int RS = rec_stride<Real, F>();
   const RenderGeom rg = geom_of(L);
   const int threads = rg.CW * rg.CH / PPT;
-  const size_t smem = (size_t)threads * (2 * RS + GS) * sizeof(Real) +
-                      32 * sizeof(Real) + (size_t)threads * 2 * sizeof(uint32_t);
+  // the records, their sums, the block scratch, an index per record, and the
+  // stage slots or (after the staging barrier) the warps' rows
+  const size_t stage = (size_t)threads * RS, rows = (size_t)(threads / 32) * row_floats<Real, GS>();
+  const size_t smem = ((size_t)threads * (RS + GS) + 32 + (stage > rows ? stage : rows)) * sizeof(Real) +
+                      (size_t)threads * sizeof(uint32_t);
   auto kernel = render_bwd_kernel<Real, F, PPT, DEPTH, WIDE>;
   static PerDeviceOnce attr;
   attr.run([&] {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                96 * 1024) == cudaSuccess;
+                                kMaxBwdSmem) == cudaSuccess;
   });
   auto* hdr = at<Header>(ws, L.off_header);
   dim3 grid(L.NT * rg.S, L.B);
