@@ -143,6 +143,20 @@ __device__ __forceinline__ void bulk_wait_read() {
 __device__ __forceinline__ void bulk_wait_all() {
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
+// One lane of a converged warp, always the same.  The MMA and load warps run
+// their loops with all lanes and let one issue: their control flow and operands
+// are then uniform, as the tensor-core and TMA instructions take them.  (With a
+// lane-0 branch around the loops every MMA's descriptors were first moved to
+// uniform registers one by one: 650 cycles to issue the four MMAs of a weight
+// block that run for 512.)
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(ok));
+  return ok != 0;
+}
+// a wait's outcome, the same for the whole warp
+__device__ __forceinline__ bool warp_ok(bool ok) { return __all_sync(0xffffffffu, ok); }
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 __device__ __forceinline__ void tc_fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
@@ -220,30 +234,30 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// 64 consecutive FP32 columns of this warp's 32 TMEM lanes: one load and one
-// wait for twice the columns of tmem_ld32 (half the exposed load latency)
-__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float* v) {
-  uint32_t r[64];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x64.b32 {"
-      "%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, "
-      "%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, "
-      "%48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%64];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
-        "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]),
-        "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]),
-        "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]),
-        "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]),
-        "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]),
-        "=r"(r[63])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+// 64 consecutive FP32 columns of this warp's 32 TMEM lanes, spread as a matrix
+// fragment: lane i's value v[32 h + 4 g + 2 s + o] is row 16 h + 8 s + i / 4,
+// column 8 g + 2 (i % 4) + o.  A lane then holds only 16 distinct columns, four
+// rows each (all 64 columns of one row with the 32x32b shape).
+__device__ __forceinline__ void tmem_ld64_frag(uint32_t taddr, float* v) {
 #pragma unroll
-  for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
+  for (int h = 0; h < 2; ++h) {
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x8.b32 {"
+        "%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+          "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
+          "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
+          "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr + ((uint32_t)(16 * h) << 16)));
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[32 * h + i] = __uint_as_float(r[i]);
+  }
+}
+__device__ __forceinline__ void tmem_wait_ld() {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ void store_row_bf16(__nv_bfloat16* dst, const float* v) {
@@ -259,28 +273,92 @@ __device__ __forceinline__ void store_row_bf16(__nv_bfloat16* dst, const float* 
   for (int i = 0; i < 4; ++i) d[i] = q[i];
 }
 
-// 32 columns [n, n + 32) of output row m
-// bf16_rn(v) > 0 for v >= 0 (or -0): v above 2^-134, half the smallest BF16
-// subnormal (ties round to even, i.e. to zero)
-__device__ __forceinline__ uint32_t relu_bits(const float* v) {
-  uint32_t bits = 0;
-#pragma unroll
-  for (int j = 0; j < 32; ++j) bits |= (v[j] > 0x1p-134f ? 1u : 0u) << j;
-  return bits;
+// ReLU masks, one bit per unit, as the fused epilogues hold a tile: per 128-row
+// tile, 32-row quarter, 64-column block and lane two words, whose halves 2 h + s
+// are the rows 16 h + 8 s + lane / 4; bit g of a half is column 8 g + 2 (lane %
+// 4), bit 8 + g the next column -- the two halves of a packed BF16 pair.  A
+// packed comparison (0xFFFF per half) enters them with one logic instruction,
+// and one shift and one byte permutation turn a pair of bits back into a mask of
+// the packed values (one compare and select per value before: 63 % more
+// instructions in the training forward than in inference).
+constexpr int kMaskTileWords = BM * kW / 32;  // 1024
+__device__ __forceinline__ size_t mask_at(int tile, int q, int cb, int lane) {
+  return (size_t)tile * kMaskTileWords + ((q * 4 + cb) * 32 + lane) * 2;
+}
+// the pair's comparison: bits g (low half) and 24 + g (high half)
+__device__ __forceinline__ uint32_t mask_add(uint32_t acc, uint32_t w, int g) {
+  const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(&w);
+  return acc | (__hgt2_mask(h, __nv_bfloat162(__float2bfloat16_rn(0.f), __float2bfloat16_rn(0.f))) &
+                (0x01000001u << g));
+}
+// two rows' comparisons to one word
+__device__ __forceinline__ uint32_t mask_word(uint32_t r0, uint32_t r1) {
+  r0 |= r0 >> 16;
+  r1 |= r1 >> 16;
+  return __byte_perm(r0, r1, 0x5410);
+}
+// 0xFFFF per packed value whose bit is set: pair g of the word's half s
+template <int S>
+__device__ __forceinline__ uint32_t mask_pair(uint32_t bits, int g) {
+  uint32_t m;  // bits g and 8 + g to the bytes' sign bits, each copied over its half
+  asm("prmt.b32 %0, %1, 0, %2;" : "=r"(m) : "r"(bits << (7 - g)), "n"(S ? 0xBBAA : 0x9988));
+  return m;
+}
+// the byte that holds row m's bits of the block's columns 2 t + odd + 8 g
+__device__ __forceinline__ uint8_t* mask_byte(uint32_t* bits, int m, int cb, int t, int odd) {
+  const int rr = m & 31;
+  uint32_t* w = bits + mask_at(m / BM, (m % BM) >> 5, cb, (rr & 7) * 4 + t) + (rr >> 4);
+  return reinterpret_cast<uint8_t*>(w) + 2 * ((rr >> 3) & 1) + odd;
+}
+// two values to packed BF16, the first in the low half
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  uint32_t w;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(hi), "f"(lo));
+  return w;
+}
+// the same with the ReLU folded into the conversion: each BF16 value is
+// bf16_rn(v) clamped at zero, which equals bf16_rn(max(v, 0))
+__device__ __forceinline__ uint32_t pack_bf16_relu(float lo, float hi) {
+  uint32_t w;
+  asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(hi), "f"(lo));
+  return w;
+}
+// two single-precision additions in one instruction, each rounded on its own
+__device__ __forceinline__ void add2(float& a, float& b, float x, float y) {
+  unsigned long long u, v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(u) : "f"(a), "f"(b));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(u) : "l"(v));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(u));
 }
 
+// 32 columns [n, n + 32) of output row m
 template <int EPI>
 __device__ __forceinline__ void epilogue(const GemmArgs& p, int m, int n, float* v) {
   if (EPI == EPI_HIDDEN || EPI == EPI_MASK) {
     if (EPI == EPI_HIDDEN) {
 #pragma unroll
       for (int j = 0; j < 32; ++j) v[j] = fmaxf(v[j] + __ldg(p.bias + n + j), 0.f);
-      p.mbits[(size_t)m * (kW / 32) + n / 32] = relu_bits(v);
-    } else {
-      const uint32_t bits = __ldg(p.mbits + (size_t)m * (kW / 32) + n / 32);
+      // columns n..n+31 are half of a block: one nibble of each of its 8 bytes
+      const int g0 = (n & 63) / 8;
 #pragma unroll
-      for (int j = 0; j < 32; ++j)
-        if (!((bits >> j) & 1u)) v[j] = 0.f;
+      for (int k = 0; k < 8; ++k) {
+        uint32_t nib = 0;
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+          nib |= (__float2bfloat16_rn(v[8 * g + k]) > __float2bfloat16_rn(0.f) ? 1u : 0u) << g;
+        uint8_t* d = mask_byte(p.mbits, m, n / 64, k >> 1, k & 1);
+        *d = g0 ? (uint8_t)(*d | (nib << 4)) : (uint8_t)nib;
+      }
+    } else {
+      const int g0 = (n & 63) / 8;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const uint32_t byte = *mask_byte(p.mbits, m, n / 64, k >> 1, k & 1) >> g0;
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+          if (!((byte >> g) & 1u)) v[8 * g + k] = 0.f;
+      }
     }
     store_row_bf16(p.out_b + (size_t)m * p.ldo + n, v);
   } else if (EPI == EPI_HEAD) {
@@ -342,7 +420,7 @@ __global__ void __launch_bounds__(192, MT == 2 ? 1 : 2)
   constexpr bool COLSUM = EPI == EPI_PARTIAL && MNA && MT == 2;
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * kStages,
                  done = full0 + 16 * kStages;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
   const int kb0 = blockIdx.z * p.kb_per_split;
   const int nkb = min(p.kb_per_split, p.kb_total - kb0);
@@ -359,24 +437,25 @@ __global__ void __launch_bounds__(192, MT == 2 ? 1 : 2)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *slot;
+  const uint32_t tmem = (uint32_t)uniform((int)*slot);
 
   if (warp == 4) {
     // TMA producer
-    if (lane == 0 && nkb > 0 && !p.inject_no_loads) {
+    if (nkb > 0 && !p.inject_no_loads) {
       int issued = 0;
       for (int i = 0; i < nkb; ++i) {
         const int s = i % kStages;
         const uint32_t ph = (uint32_t)(i / kStages) & 1u;
-        if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, p.status, p.wait_ns)) break;
-        mbar_expect_tx(full0 + 8 * s, STAGE);
-        const uint32_t sa = sbase + s * STAGE;
-        if (MNA) {
+        if (!warp_ok(mbar_wait(empty0 + 8 * s, ph ^ 1u, p.status, p.wait_ns))) break;
+        if (elect_one()) {
+          mbar_expect_tx(full0 + 8 * s, STAGE);
+          const uint32_t sa = sbase + s * STAGE;
+          if (MNA) {
 #pragma unroll
-          for (int j = 0; j < 2 * MT; ++j)
-            tma_load_2d(sa + j * 8192, &tmA, full0 + 8 * s, m0 * MT + 64 * j, (kb0 + i) * BK);
-        } else {
-          tma_load_2d(sa, &tmA, full0 + 8 * s, (kb0 + i) * BK, m0 * MT);
+            for (int j = 0; j < 2 * MT; ++j)
+              tma_load_2d(sa + j * 8192, &tmA, full0 + 8 * s, m0 * MT + 64 * j, (kb0 + i) * BK);
+          } else {
+            tma_load_2d(sa, &tmA, full0 + 8 * s, (kb0 + i) * BK, m0 * MT);
         }
         if (MNB) {
 #pragma unroll
@@ -386,6 +465,8 @@ __global__ void __launch_bounds__(192, MT == 2 ? 1 : 2)
         } else {
           tma_load_2d(sa + A_BYTES, &tmB, full0 + 8 * s, (kb0 + i) * BK, n0);
         }
+        }
+        __syncwarp();
         issued = i + 1;
       }
       // every load issued has landed before the CTA may exit
@@ -394,27 +475,31 @@ __global__ void __launch_bounds__(192, MT == 2 ? 1 : 2)
     }
   } else if (warp == 5) {
     // MMA issuer
-    if (lane == 0 && nkb > 0) {
+    if (nkb > 0) {
       constexpr uint32_t idesc = idesc_bf16(BM, BN, MNA, MNB);
       for (int i = 0; i < nkb; ++i) {
         const int s = i % kStages;
         const uint32_t ph = (uint32_t)(i / kStages) & 1u;
-        if (!mbar_wait(full0 + 8 * s, ph, p.status, p.wait_ns)) break;
+        if (!warp_ok(mbar_wait(full0 + 8 * s, ph, p.status, p.wait_ns))) break;
         tc_fence_after();
-        const uint32_t sa = sbase + s * STAGE, sb = sa + A_BYTES;
+        if (elect_one()) {
+          const uint32_t sa = sbase + s * STAGE, sb = sa + A_BYTES;
 #pragma unroll
-        for (int k = 0; k < BK / 16; ++k)
+          for (int k = 0; k < BK / 16; ++k)
 #pragma unroll
-          for (int t = 0; t < MT; ++t) {
-            // K step of 16: 32 bytes along a K-major row, two 8-row groups MN-major
-            const uint64_t da = MNA ? sw128_mn_desc(sa + t * 16384 + 2048 * k)
-                                    : sw128_desc(sa + t * BM * 128 + 32 * k);
-            const uint64_t db = MNB ? sw128_mn_desc(sb + 2048 * k) : sw128_desc(sb + 32 * k);
-            umma_bf16(tmem + (uint32_t)(t * BN), da, db, idesc, (i > 0 || k > 0) ? 1u : 0u);
-          }
-        umma_commit(empty0 + 8 * s);
+            for (int t = 0; t < MT; ++t) {
+              // K step of 16: 32 bytes along a K-major row, two 8-row groups MN-major
+              const uint64_t da = MNA ? sw128_mn_desc(sa + t * 16384 + 2048 * k)
+                                      : sw128_desc(sa + t * BM * 128 + 32 * k);
+              const uint64_t db = MNB ? sw128_mn_desc(sb + 2048 * k) : sw128_desc(sb + 32 * k);
+              umma_bf16(tmem + (uint32_t)(t * BN), da, db, idesc, (i > 0 || k > 0) ? 1u : 0u);
+            }
+          umma_commit(empty0 + 8 * s);
+        }
+        __syncwarp();
       }
-      umma_commit(done);  // completes once every MMA issued above has
+      if (elect_one()) umma_commit(done);  // completes once every MMA issued above has
+      __syncwarp();
     }
   } else {
     float cs0 = 0.f, cs1 = 0.f;  // COLSUM: columns 2 tid, 2 tid + 1 of A
@@ -563,75 +648,97 @@ __global__ void mlp_encode_kernel(const float* __restrict__ means, Times tm, int
   for (int q = 0; q < kIn / 32; ++q) store_row_bf16(enc + (size_t)m * kIn + 32 * q, e + 32 * q);
 }
 
-// dL/d(delta) fp32 [M][3] -> bf16 [M_pad][32] and its transpose [32][M_pad]
-// (and the head's bias gradient, the column sums of the rounded values)
-__global__ void __launch_bounds__(128)
+// dL/d(delta) fp32 [M][3] -> BF16, transposed: [3][M_pad] (the head's weight
+// gradient reduces over the rows) and, for the one-GEMM-per-layer chain only,
+// row-major [M_pad][32] (dz, else null); and the head's bias gradient, the
+// column sums of the rounded values.  Rows 3..31 of the transposed array are
+// beyond its tensor map and arrive as zeros.  The column sums go through the
+// CTA first: with one atomic per warp and column the 28k additions to three
+// addresses serialised (19.7 us at 300k rows).
+constexpr int kHeadGradThreads = 256;
+__global__ void __launch_bounds__(kHeadGradThreads)
     mlp_head_grad_kernel(const float* __restrict__ dd, int M, int M_pad,
                          __nv_bfloat16* __restrict__ dz, __nv_bfloat16* __restrict__ dzt,
                          float* __restrict__ dbias, int ldb) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  float v[32];
+  __shared__ float s_sum[kHeadGradThreads / 32][3];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float sum[3] = {0.f, 0.f, 0.f};
+  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M_pad; m += gridDim.x * blockDim.x) {
+    __nv_bfloat16 q[3];
 #pragma unroll
-  for (int j = 0; j < 32; ++j) v[j] = 0.f;
-  if (m < M) {
+    for (int j = 0; j < 3; ++j) {
+      q[j] = __float2bfloat16_rn(m < M ? dd[(size_t)m * 3 + j] : 0.f);
+      dzt[(size_t)j * M_pad + m] = q[j];
+      sum[j] += __bfloat162float(q[j]);
+    }
+    if (dz) {
+      float v[32];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) v[j] = dd[(size_t)m * 3 + j];
-  }
-  if (m < M_pad) {
-    store_row_bf16(dz + (size_t)m * kHeadRows, v);
-#pragma unroll
-    for (int j = 0; j < kHeadRows; ++j) dzt[(size_t)j * M_pad + m] = __float2bfloat16_rn(v[j]);
+      for (int j = 0; j < 32; ++j) v[j] = j < 3 ? __bfloat162float(q[j]) : 0.f;
+      store_row_bf16(dz + (size_t)m * kHeadRows, v);
+    }
   }
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    float b = __bfloat162float(__float2bfloat16_rn(v[j]));
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
-    if ((threadIdx.x & 31) == 0 && b != 0.f) atomicAdd(dbias + (size_t)j * ldb, b);
+    for (int o = 16; o > 0; o >>= 1) sum[j] += __shfl_xor_sync(0xffffffffu, sum[j], o);
+    if (lane == 0) s_sum[w][j] = sum[j];
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    float b = 0.f;
+    for (int k = 0; k < kHeadGradThreads / 32; ++k) b += s_sum[k][threadIdx.x];
+    if (b != 0.f) atomicAdd(dbias + (size_t)threadIdx.x * ldb, b);
   }
 }
 
 // dL/d(means) from the encoding's gradient (the position part, columns
-// 0..62), summed over the frames: one warp per Gaussian.  The frames' rows
-// are summed first (coalesced, lanes over columns), then each lane applies
-// the derivative of its columns' encoding -- d sin(f pi x)/dx = f pi cos(f pi x),
-// d cos(f pi x)/dx = -f pi sin(f pi x) -- and the warp reduces per axis.
-__global__ void __launch_bounds__(256)
+// 0..62), summed over the frames: two threads per Gaussian, thread h taking the
+// bands 5 h .. 5 h + 4 (columns 30 h + 3 .. 30 h + 32) and thread 0 the position
+// itself.  The frames' rows are summed first, then the derivative of the
+// encoding is applied -- d sin(f pi x)/dx = f pi cos(f pi x), d cos(f pi x)/dx =
+// -f pi sin(f pi x).  One warp per Gaussian (a column per lane) evaluated every
+// sine-cosine pair twice and spent 15 shuffles per Gaussian: 70 us at 300k
+// Gaussians, bound by instruction issue at 1.1 TB/s.
+__global__ void __launch_bounds__(128)
     mlp_encode_bwd_kernel(const float* __restrict__ means, const float* __restrict__ denc, int N,
                           int B, float inv_scale, float* __restrict__ dmeans) {
-  const int g = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (g >= N) return;
-  float d0 = 0.f, d1 = 0.f;  // columns lane and lane + 32, summed over the frames
-  for (int b = 0; b < B; ++b) {
-    const float* row = denc + ((size_t)b * N + g) * kIn;
-    d0 += __ldg(row + lane);
-    if (lane < 31) d1 += __ldg(row + 32 + lane);
-  }
-  float acc[3] = {0.f, 0.f, 0.f};
+  constexpr int kBands = kFreq / 2, kCols = 6 * kBands + 4;  // (even: float2 loads)
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int g = min(i >> 1, N - 1), h = i & 1;  // (a whole warp reaches the shuffles)
+  float d[kCols];
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int c = lane + 32 * h;
-    const float d = h ? d1 : d0;
-    if (c < 3) {
-      acc[c] += d;
-    } else if (c < 63) {
-      const int l = (c - 3) / 6, w = (c - 3) - 6 * l, a = w < 3 ? w : w - 3;
-      const float f = (float)(1 << l);
-      const float x = __ldg(means + (size_t)g * 3 + a) * inv_scale;
+  for (int c = 0; c < kCols; ++c) d[c] = 0.f;
+#pragma unroll 2
+  for (int b = 0; b < B; ++b) {
+    const float2* row =
+        reinterpret_cast<const float2*>(denc + ((size_t)b * N + g) * kIn + 6 * kBands * h);
+#pragma unroll
+    for (int c = 0; c < kCols / 2; ++c) {
+      const float2 v = __ldg(row + c);
+      d[2 * c] += v.x;
+      d[2 * c + 1] += v.y;
+    }
+  }
+  float acc[3], x[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    acc[a] = h ? 0.f : d[a];
+    x[a] = __ldg(means + (size_t)g * 3 + a) * inv_scale;
+  }
+  float f = h ? (float)(1 << kBands) : 1.f;
+#pragma unroll
+  for (int l = 0; l < kBands; ++l, f *= 2.f) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
       float sn, cs;
-      sincospif(f * x, &sn, &cs);
-      const float term = f * 3.14159265358979323846f * (w < 3 ? cs * d : -sn * d);
-      acc[0] += a == 0 ? term : 0.f;
-      acc[1] += a == 1 ? term : 0.f;
-      acc[2] += a == 2 ? term : 0.f;
+      sincospif(f * x[a], &sn, &cs);
+      acc[a] += f * 3.14159265358979323846f * (cs * d[3 + 6 * l + a] - sn * d[6 + 6 * l + a]);
     }
   }
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], off);
-  if (lane == 0)
+  for (int a = 0; a < 3; ++a) acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], 1);
+  if (h == 0 && (i >> 1) < N)
     for (int a = 0; a < 3; ++a) dmeans[(size_t)g * 3 + a] = acc[a] * inv_scale;
 }
 
@@ -665,16 +772,34 @@ __global__ void mlp_unpack_grads_kernel(const float* __restrict__ dwx, float* __
   }
 }
 
-// sum of the row-split partials [splits][256][K] -> dW block [256][ld]
-__global__ void mlp_reduce_dw_kernel(const float* __restrict__ part, int splits, int K,
-                                     float* __restrict__ dw, int ld) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= kW * K) return;
+// sum of the row-split partials [splits][256][K] -> dW block [256][ld]: a CTA
+// takes 32 groups of four consecutive values, its eight warps every eighth
+// split each (the partials lie in L2; with one value per thread and all splits
+// in a row the loads in flight bounded it: 13.5 us per layer of 152 splits)
+constexpr int kReduceWarps = 8;
+__global__ void __launch_bounds__(32 * kReduceWarps)
+    mlp_reduce_dw_kernel(const float* __restrict__ part, int splits, int K,
+                         float* __restrict__ dw, int ld) {
+  __shared__ float4 s_sum[kReduceWarps][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int e = (blockIdx.x * 32 + lane) * 4;  // 256 K is a multiple of 128
   const size_t stride = (size_t)kW * K;
-  float s = 0.f;
-  for (int z = 0; z < splits; ++z) s += part[(size_t)z * stride + e];
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 5
+  for (int z = w; z < splits; z += kReduceWarps) {
+    const float4 v = __ldcs(reinterpret_cast<const float4*>(part + (size_t)z * stride + e));
+    s.x += v.x, s.y += v.y, s.z += v.z, s.w += v.w;
+  }
+  s_sum[w][lane] = s;
+  __syncthreads();
+  if (w != 0) return;
+#pragma unroll
+  for (int k = 1; k < kReduceWarps; ++k) {
+    const float4 v = s_sum[k][lane];
+    s.x += v.x, s.y += v.y, s.z += v.z, s.w += v.w;
+  }
   const int o = e / K, i = e - o * K;
-  dw[(size_t)o * ld + i] = s;
+  *reinterpret_cast<float4*>(dw + (size_t)o * ld + i) = s;
 }
 
 // ---- fused forward (inference): all layers of 128-row tiles in one CTA -------
@@ -691,7 +816,8 @@ constexpr int kFusedStages = 3;
 constexpr int kPair = 2;                   // tiles in flight per CTA
 constexpr int kActBytes = BM * kW * 2;     // 64 KB per tile
 constexpr int kWStageBytes = kW * BK * 2;  // 32 KB (a 256-row k-block of W)
-constexpr int kFusedSmem = kPair * kActBytes + kFusedStages * kWStageBytes + 1024 + 256;
+// (the barriers' 256 bytes, one layer's biases, and the alignment)
+constexpr int kFusedSmem = kPair * kActBytes + kFusedStages * kWStageBytes + 256 + kW * 4 + 1024;
 
 struct FusedMaps {
   CUtensorMap w[kDepth + 1];  // bf16 W of the hidden layers (256 rows), head (32 rows)
@@ -707,40 +833,133 @@ __device__ __forceinline__ uint32_t act_off(int r, int c) {
   return (uint32_t)(kb * 16384 + (r >> 3) * 1024 + (r & 7) * 128 +
                     ((((cc >> 3) ^ (r & 7)) << 4) | ((cc & 7) << 1)));
 }
-__device__ __forceinline__ void store_act32(uint8_t* act, int r, int c, const float* v) {
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    uint4 u;
-    uint32_t* w = reinterpret_cast<uint32_t*>(&u);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      __nv_bfloat162 h = __floats2bfloat162_rn(v[8 * q + 2 * i], v[8 * q + 2 * i + 1]);
-      w[i] = *reinterpret_cast<uint32_t*>(&h);
-    }
-    *reinterpret_cast<uint4*>(act + act_off(r, c + 8 * q)) = u;
-  }
+__device__ __forceinline__ void store_act8(uint8_t* act, int r, int c, const float* v) {
+  *reinterpret_cast<uint4*>(act + act_off(r, c)) =
+      make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
+                 pack_bf16(v[6], v[7]));
+}
+__device__ __forceinline__ void store_act16(uint8_t* act, int r, int c, const float* v) {
+  store_act8(act, r, c, v);
+  store_act8(act, r, c + 8, v + 8);
 }
 
-// the same with the ReLU folded into the conversion: each BF16 value is
-// bf16_rn(v) clamped at zero, which equals bf16_rn(max(v, 0))
-__device__ __forceinline__ void store_act32_relu(uint8_t* act, int r, int c, const float* v) {
+// A lane's part of the address of a fragment's store into an activation tile: a
+// stmatrix of four 8 x 8 matrices (column groups g, g + 1 of rows 0..7 and 8..15 of
+// a 16-row half) takes the matrices' row addresses from the lanes in order.
+struct FragStore {
+  uint32_t row;  // shared address of the lane's row, first chunk of block 0
+  uint32_t x;    // the swizzle and the lane's column group, to be XORed with 16 g
+};
+__device__ __forceinline__ FragStore frag_store(uint32_t act_s, int q, int lane) {
+  const int r = q * 32 + ((lane >> 3) & 1) * 8 + (lane & 7);
+  return {act_s + (uint32_t)((r >> 3) * 1024 + (r & 7) * 128),
+          (uint32_t)(((lane >> 4) ^ (lane & 7)) << 4)};
+}
+// packed values of column groups g, g + 1 (g even) of 16-row half h, block cb
+__device__ __forceinline__ void store_frag(const FragStore& f, int cb, int h, int g, uint32_t a0,
+                                           uint32_t a1, uint32_t b0, uint32_t b1) {
+  const uint32_t at = f.row + (uint32_t)(cb * 16384 + h * 2048) + (f.x ^ (uint32_t)(16 * g));
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(at),
+               "r"(a0), "r"(a1), "r"(b0), "r"(b1)
+               : "memory");
+}
+
+// encode_row's values of columns [C0, C0 + 16) from the scaled position (columns
+// below 63)
+template <int C0>
+__device__ __forceinline__ void encode16(const float* x, float* e) {
+  float f = 1.f;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    uint4 u;
-    uint32_t* w = reinterpret_cast<uint32_t*>(&u);
+  for (int l = 0; l < kFreq; ++l, f *= 2.f)
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;"
-          : "=r"(w[i])
-          : "f"(v[8 * q + 2 * i + 1]), "f"(v[8 * q + 2 * i]));
-    *reinterpret_cast<uint4*>(act + act_off(r, c + 8 * q)) = u;
+    for (int a = 0; a < 3; ++a) {
+      if (l == 0 && a >= C0 && a < C0 + 16) e[a - C0] = x[a];
+      const int cs = 3 + 6 * l + a, cc = cs + 3;
+      const bool is = cs >= C0 && cs < C0 + 16, ic = cc >= C0 && cc < C0 + 16;
+      if (is || ic) {
+        float sn, co;
+        sincospif(f * x[a], &sn, &co);
+        if (is) e[cs - C0] = sn;
+        if (ic) e[cc - C0] = co;
+      }
+    }
+}
+
+// encode_row's values of one row, straight into the row's place in the tile, by
+// four threads: part p takes the position's columns 16 p .. 16 p + 15, part 0
+// also the time's (64..83), the others the zeros behind them.  The time's values
+// depend on the frame only: where a warp's rows lie in one frame, ten lanes
+// evaluate one band each and the warp shares them.  (One thread per row, 40
+// sine-cosine pairs: the tensor cores idled through them.)
+__device__ __forceinline__ void encode_part(const float* __restrict__ means, const Times& tm,
+                                            int N, int M, float inv_scale, int m, int part,
+                                            uint8_t* act, int r) {
+  const bool in = m < M;
+  const int b = in ? m / N : 0, g = in ? m - b * N : 0;
+  const float t = tm.t[b];
+  float x[3], e[32];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) x[a] = in ? means[(size_t)g * 3 + a] * inv_scale : 0.f;
+  if (part == 0) {
+    encode16<0>(x, e);
+  } else if (part == 1) {
+    encode16<16>(x, e);
+  } else if (part == 2) {
+    encode16<32>(x, e);
+  } else {
+    encode16<48>(x, e);
+    e[15] = t;
   }
+#pragma unroll
+  for (int c = 0; c < 16; ++c) e[c] = in ? e[c] : 0.f;
+  store_act16(act, r, 16 * part, e);
+  if (part != 0) {  // columns 80..127: the last bands' four are part 0's
+    uint4* z = reinterpret_cast<uint4*>(act + act_off(r, 80 + 16 * (part - 1)));
+    if (part > 1) *z = make_uint4(0, 0, 0, 0);
+    *reinterpret_cast<uint4*>(act + act_off(r, 88 + 16 * (part - 1))) = make_uint4(0, 0, 0, 0);
+    return;
+  }
+  float te[24], sn, cs;
+  const int lane = threadIdx.x & 31;
+  const int b0 = __shfl_sync(0xffffffffu, b, 0);
+  if (__all_sync(0xffffffffu, b == b0 || !in)) {
+    sincospif((float)(1 << (lane < kFreq ? lane : 0)) * tm.t[b0], &sn, &cs);
+#pragma unroll
+    for (int l = 0; l < kFreq; ++l) {
+      te[2 * l] = __shfl_sync(0xffffffffu, sn, l);
+      te[2 * l + 1] = __shfl_sync(0xffffffffu, cs, l);
+    }
+  } else {
+    float f = 1.f;
+#pragma unroll
+    for (int l = 0; l < kFreq; ++l, f *= 2.f) sincospif(f * t, &te[2 * l], &te[2 * l + 1]);
+  }
+#pragma unroll
+  for (int c = 0; c < 24; ++c) te[c] = c < 2 * kFreq && in ? te[c] : 0.f;
+  store_act16(act, r, 64, te);
+  store_act8(act, r, 80, te + 16);
 }
 
 // warps 0-7: epilogue (warp w: TMEM lanes / rows 32 (w % 4) .. + 31, columns
-// 128 (w / 4) .. + 127); warp 8: TMA; warp 9: MMA
+// 128 (w / 4) .. + 127); warp 8: TMA; warp 9: MMA.
+// What bounds the fused kernels is the 128 bytes a cycle that shared memory (and
+// the L1 data path behind every load) moves: for a tile's layer the MMAs read
+// 192 KB of operands (1536 cycles for 2048 of MMA), the weights arrive with 128 KB
+// and the epilogue stores 64 KB.  So the epilogue takes the accumulators as matrix
+// fragments (a lane: 16 columns of four rows), which needs a quarter of the bias
+// values per lane that one row of 64 columns did (those alone took 1024 cycles
+// per tile and layer, from global or shared memory alike), and stores them by
+// stmatrix.  300k rows of inference: 260 -> 191 us, 0.77 of the measured BF16
+// peak (timelines: 3300 -> 2300 cycles per tile and layer); training forward
+// 392 -> 319 us.  Sixteen epilogue warps measured the same.
 constexpr int kFusedEpiWarps = 8;
-constexpr int kFusedThreads = 32 * (kFusedEpiWarps + 2);
+constexpr int kFusedEpiThreads = 32 * kFusedEpiWarps;
+constexpr int kFusedThreads = kFusedEpiThreads + 64;
+constexpr int kParts = kFusedEpiWarps / 4;       // warps that share a row
+constexpr int kBlocks = kW / 64 / kParts;        // 64-column blocks of a thread
+__device__ __forceinline__ void epi_sync() {
+  asm volatile("bar.sync 1, %0;" ::"n"(kFusedEpiThreads) : "memory");
+}
 
 // What a training forward keeps for the backward (TRAIN): the encoded input
 // and every hidden activation (row-major BF16, stored by TMA from the tile in
@@ -767,10 +986,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
   // bars: full[S], empty[S], acc_ready[kPair], act_ready[kPair]
   uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 2 * kFusedStages + 2 * kPair);
   int* s_ok = reinterpret_cast<int*>(slot + 1);  // the epilogue's shared wait outcome
+  float* s_bias = reinterpret_cast<float*>(bars + 32);  // the layer's biases
   const uint32_t act_s = smem_u32(smem), w_s = act_s + kPair * kActBytes;
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * kFusedStages;
   const uint32_t acc0 = full0 + 16 * kFusedStages, actr0 = acc0 + 8 * kPair;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int n_pairs = (n_tiles + kPair - 1) / kPair;
   if (threadIdx.x == 0) {
     for (int i = 0; i < kFusedStages; ++i) {
@@ -787,11 +1007,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *slot;
+  const uint32_t tmem = (uint32_t)uniform((int)*slot);
 
   if (warp == kFusedEpiWarps) {
     // weights of every (layer, tile) item, k-block by k-block
-    if (lane == 0 && !inject_no_loads) {
+    if (!inject_no_loads) {
       int it = 0;
       bool ok = true;
       for (int pr = blockIdx.x; ok && pr < n_pairs; pr += gridDim.x)
@@ -801,11 +1021,13 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
             const uint32_t bytes = (uint32_t)(l == kDepth ? kHeadRows : kW) * BK * 2;
             for (int kb = 0; kb < nkb; ++kb, ++it) {
               const int s = it % kFusedStages;
-              if (!(ok = mbar_wait(empty0 + 8 * s, ((uint32_t)(it / kFusedStages) & 1u) ^ 1u,
-                                   status, wait_ns)))
+              if (!(ok = warp_ok(mbar_wait(empty0 + 8 * s, ((uint32_t)(it / kFusedStages) & 1u) ^ 1u,
+                                           status, wait_ns))))
                 break;
-              mbar_expect_tx(full0 + 8 * s, bytes);
-              tma_load_2d(w_s + s * kWStageBytes, &maps.w[l], full0 + 8 * s, kb * BK, 0);
+              if (elect_one()) {
+                mbar_expect_tx(full0 + 8 * s, bytes);
+                tma_load_2d(w_s + s * kWStageBytes, &maps.w[l], full0 + 8 * s, kb * BK, 0);
+              }
             }
           }
       // every load issued has landed before the CTA may exit
@@ -814,14 +1036,14 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
                   wait_ns);
     }
   } else if (warp == kFusedEpiWarps + 1) {
-    if (lane == 0) {
+    {
       int it = 0;
       uint32_t act_ph[kPair] = {0, 0};
       bool ok = true;
       for (int pr = blockIdx.x; ok && pr < n_pairs; pr += gridDim.x)
         for (int l = 0; ok && l <= kDepth; ++l)
           for (int t = 0; ok && t < kPair; ++t) {
-            if (!(ok = mbar_wait(actr0 + 8 * t, act_ph[t], status, wait_ns))) break;
+            if (!(ok = warp_ok(mbar_wait(actr0 + 8 * t, act_ph[t], status, wait_ns)))) break;
             act_ph[t] ^= 1u;
             tc_fence_after();
             const int nkb = (l == 0 ? kIn : kW) / BK;
@@ -829,38 +1051,38 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
             const uint32_t d = tmem + (uint32_t)(t * kW);
             for (int kb = 0; kb < nkb; ++kb, ++it) {
               const int s = it % kFusedStages;
-              if (!(ok = mbar_wait(full0 + 8 * s, (uint32_t)(it / kFusedStages) & 1u, status,
-                                   wait_ns)))
+              if (!(ok = warp_ok(mbar_wait(full0 + 8 * s, (uint32_t)(it / kFusedStages) & 1u, status,
+                                           wait_ns))))
                 break;
               tc_fence_after();
               const uint32_t sa = act_s + t * kActBytes + kb * 16384, sb = w_s + s * kWStageBytes;
+              if (elect_one()) {
 #pragma unroll
-              for (int k = 0; k < BK / 16; ++k)
-                umma_bf16(d, sw128_desc(sa + 32 * k), sw128_desc(sb + 32 * k), idesc,
-                          (kb > 0 || k > 0) ? 1u : 0u);
-              umma_commit(empty0 + 8 * s);
+                for (int k = 0; k < BK / 16; ++k)
+                  umma_bf16(d, sw128_desc(sa + 32 * k), sw128_desc(sb + 32 * k), idesc,
+                            (kb > 0 || k > 0) ? 1u : 0u);
+                umma_commit(empty0 + 8 * s);
+              }
+              __syncwarp();
             }
-            umma_commit(acc0 + 8 * t);
+            if (elect_one()) umma_commit(acc0 + 8 * t);
+            __syncwarp();
           }
     }
   } else {
-    // epilogue warps: row r of every tile, one half of the columns
-    const int q = warp & 3, half = warp >> 2;
+    // epilogue warps: row r of every tile, a quarter of the columns
+    const int q = warp & 3, part = warp >> 2;
     const int r = q * 32 + lane;
     uint32_t acc_ph[kPair] = {0, 0};
     bool ok = true;
     for (int pr = blockIdx.x; ok && pr < n_pairs; pr += gridDim.x) {
       for (int t = 0; t < kPair; ++t) {
-        if (half == 0) {
-          float e[kIn];
-          const int m = (pr * kPair + t) * BM + r;
-          encode_row(means, tm, N, M, inv_scale, m, e);
-          uint8_t* act = smem + t * kActBytes;
-#pragma unroll
-          for (int c = 0; c < kIn; c += 32) store_act32(act, r, c, e + c);
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        }
-        asm volatile("bar.sync 1, 256;" ::: "memory");
+#pragma unroll 1
+        for (int k = 0; k < kBlocks; ++k)
+          encode_part(means, tm, N, M, inv_scale, (pr * kPair + t) * BM + r, part + k * kParts,
+                      smem + t * kActBytes, r);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        epi_sync();
         if (threadIdx.x == 0) mbar_arrive(actr0 + 8 * t);
         if (TRAIN && threadIdx.x == 32 * t && pr * kPair + t < n_tiles) {
           for (int kb = 0; kb < kIn / BK; ++kb)
@@ -869,51 +1091,60 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
           bulk_commit();
         }
       }
+      // (every thread is past the last pair's barrier, so its biases are free)
+      if (threadIdx.x < kW) s_bias[threadIdx.x] = __ldg(theta + bias_off_dev(0) + threadIdx.x);
       for (int l = 0; ok && l <= kDepth; ++l)
         for (int t = 0; t < kPair; ++t) {
           // one thread waits, the other epilogue threads follow the barrier, so
-          // that all 128 take the same branch (no split at the named barriers)
+          // that all of them take the same branch (no split at the named barriers)
           if (threadIdx.x == 0)
             *s_ok = mbar_wait(acc0 + 8 * t, acc_ph[t], status, wait_ns) ? 1 : 0;
           // the tile's last store has read it before it is written again
           if (TRAIN && threadIdx.x == 32 * t) bulk_wait_read();
-          asm volatile("bar.sync 1, 256;" ::: "memory");
+          epi_sync();
           // (every step ends at a named barrier that all epilogue threads reach
           // after reading the flag, so thread 0 rewrites it only afterwards)
           if (!(ok = *s_ok != 0)) break;
           acc_ph[t] ^= 1u;
           tc_fence_after();
           const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(t * kW);
-          uint8_t* act = smem + t * kActBytes;
           if (l < kDepth) {
-            const float* bias = theta + bias_off_dev(l);
+            const FragStore fs = frag_store(act_s + t * kActBytes, q, lane);
 #pragma unroll 1
-            for (int c0 = half * (kW / 2); c0 < (half + 1) * (kW / 2); c0 += 64) {
-              float vv[64];
-              tmem_ld64(trow + (uint32_t)c0, vv);
+            for (int k = 0; k < kBlocks; ++k) {
+              const int cb = part * kBlocks + k;
+              float v[64];
+              tmem_ld64_frag(trow + (uint32_t)(cb * 64), v);
+              float2 b[8];
 #pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                float* v = vv + 32 * h;
-                const int c = c0 + 32 * h;
-                const float4* b4 = reinterpret_cast<const float4*>(bias + c);
+              for (int g = 0; g < 8; ++g)
+                b[g] = *reinterpret_cast<const float2*>(s_bias + cb * 64 + 8 * g + 2 * (lane & 3));
+              tmem_wait_ld();
+              uint32_t rows[4] = {0, 0, 0, 0};
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                  const float4 b = __ldg(b4 + j);
-                  v[4 * j] += b.x;
-                  v[4 * j + 1] += b.y;
-                  v[4 * j + 2] += b.z;
-                  v[4 * j + 3] += b.w;
+              for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int g = 0; g < 8; g += 2) {
+                  uint32_t w[4];
+#pragma unroll
+                  for (int i = 0; i < 4; ++i) {  // group g + i / 2, rows 8 (i % 2)
+                    float* e = v + 32 * h + 4 * (g + (i >> 1)) + 2 * (i & 1);
+                    add2(e[0], e[1], b[g + (i >> 1)].x, b[g + (i >> 1)].y);
+                    w[i] = pack_bf16_relu(e[0], e[1]);
+                    if (TRAIN)
+                      rows[2 * h + (i & 1)] = mask_add(rows[2 * h + (i & 1)], w[i], g + (i >> 1));
+                  }
+                  store_frag(fs, cb, h, g, w[0], w[1], w[2], w[3]);
                 }
-                store_act32_relu(act, r, c, v);  // (the mask bits below: v > 2^-134
-                                                 // before or after the ReLU alike)
-                const int m = (pr * kPair + t) * BM + r;
-                if (TRAIN && m < keep.Mp)
-                  keep.bits[((size_t)l * keep.Mp + m) * (kW / 32) + c / 32] = relu_bits(v);
-              }
+              const int tile = pr * kPair + t;
+              if (TRAIN && tile < n_tiles)
+                *reinterpret_cast<uint2*>(keep.bits + (size_t)l * keep.Mp * (kW / 32) +
+                                          mask_at(tile, q, cb, lane)) =
+                    make_uint2(mask_word(rows[0], rows[1]), mask_word(rows[2], rows[3]));
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             tc_fence_before();
-            asm volatile("bar.sync 1, 256;" ::: "memory");
+            epi_sync();
             if (threadIdx.x == 0) mbar_arrive(actr0 + 8 * t);
             if (TRAIN && threadIdx.x == 32 * t && pr * kPair + t < n_tiles) {
               for (int kb = 0; kb < kW / BK; ++kb)
@@ -921,8 +1152,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
                              l * keep.Mp + (pr * kPair + t) * BM);
               bulk_commit();
             }
+            // both tiles have taken this layer's bias: the next one's
+            if (t == kPair - 1 && l + 1 < kDepth && threadIdx.x < kW)
+              s_bias[threadIdx.x] = __ldg(theta + bias_off_dev(l + 1) + threadIdx.x);
           } else {
-            if (half == 0) {
+            if (part == 0) {
               float v[32];
               tmem_ld32(trow, v);
               const float* bias = theta + head_bias_off_dev();
@@ -931,7 +1165,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
                 for (int j = 0; j < 3; ++j) delta[(size_t)m * 3 + j] = v[j] + __ldg(bias + j);
             }
             tc_fence_before();
-            asm volatile("bar.sync 1, 256;" ::: "memory");  // TMEM drained before the next pair
+            epi_sync();  // TMEM drained before the next pair
           }
         }
     }
@@ -976,7 +1210,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
   const uint32_t act_s = smem_u32(smem), w_s = act_s + kPair * kActBytes;
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * kBwdStages;
   const uint32_t acc0 = full0 + 16 * kBwdStages, actr0 = acc0 + 8 * kPair;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int n_pairs = (a.n_tiles + kPair - 1) / kPair;
   constexpr int kSteps = kDepth + 1;
   if (threadIdx.x == 0) {
@@ -994,11 +1228,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *slot;
+  const uint32_t tmem = (uint32_t)uniform((int)*slot);
 
   if (warp == kFusedEpiWarps) {
     // W^T of the head (step 0) and of layers 7..0 (steps 1..8)
-    if (lane == 0 && !inject_no_loads) {
+    if (!inject_no_loads) {
       int it = 0;
       bool ok = true;
       for (int pr = blockIdx.x; ok && pr < n_pairs; pr += gridDim.x)
@@ -1007,12 +1241,14 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
             const int nkb = st == 0 ? 1 : kW / BK;
             for (int kb = 0; kb < nkb; ++kb, ++it) {
               const int s = it % kBwdStages;
-              if (!(ok = mbar_wait(empty0 + 8 * s, ((uint32_t)(it / kBwdStages) & 1u) ^ 1u,
-                                   status, wait_ns)))
+              if (!(ok = warp_ok(mbar_wait(empty0 + 8 * s, ((uint32_t)(it / kBwdStages) & 1u) ^ 1u,
+                                           status, wait_ns))))
                 break;
-              mbar_expect_tx(full0 + 8 * s, (uint32_t)kWStageBytes);
-              tma_load_2d(w_s + s * kWStageBytes, &maps.w[st == 0 ? kDepth : kDepth - st],
-                          full0 + 8 * s, kb * BK, 0);
+              if (elect_one()) {
+                mbar_expect_tx(full0 + 8 * s, (uint32_t)kWStageBytes);
+                tma_load_2d(w_s + s * kWStageBytes, &maps.w[st == 0 ? kDepth : kDepth - st],
+                            full0 + 8 * s, kb * BK, 0);
+              }
             }
           }
       for (int i = it - kBwdStages < 0 ? 0 : it - kBwdStages; i < it; ++i)
@@ -1020,7 +1256,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
                   wait_ns);
     }
   } else if (warp == kFusedEpiWarps + 1) {
-    if (lane == 0) {
+    {
       int it = 0;
       uint32_t act_ph[kPair] = {0, 0};
       bool ok = true;
@@ -1028,39 +1264,50 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
       for (int pr = blockIdx.x; ok && pr < n_pairs; pr += gridDim.x)
         for (int st = 0; ok && st < kSteps; ++st)
           for (int t = 0; ok && t < kPair; ++t) {
-            if (!(ok = mbar_wait(actr0 + 8 * t, act_ph[t], status, wait_ns))) break;
+            if (!(ok = warp_ok(mbar_wait(actr0 + 8 * t, act_ph[t], status, wait_ns)))) break;
             act_ph[t] ^= 1u;
             tc_fence_after();
             const int nkb = st == 0 ? 1 : kW / BK;
             const uint32_t d = tmem + (uint32_t)(t * kW);
             for (int kb = 0; kb < nkb; ++kb, ++it) {
               const int s = it % kBwdStages;
-              if (!(ok = mbar_wait(full0 + 8 * s, (uint32_t)(it / kBwdStages) & 1u, status,
-                                   wait_ns)))
+              if (!(ok = warp_ok(mbar_wait(full0 + 8 * s, (uint32_t)(it / kBwdStages) & 1u, status,
+                                           wait_ns))))
                 break;
               tc_fence_after();
               const uint32_t sa = act_s + t * kActBytes + kb * 16384, sb = w_s + s * kWStageBytes;
+              if (elect_one()) {
 #pragma unroll
-              for (int k = 0; k < BK / 16; ++k)
-                umma_bf16(d, sw128_desc(sa + 32 * k), sw128_desc(sb + 32 * k), idesc,
-                          (kb > 0 || k > 0) ? 1u : 0u);
-              umma_commit(empty0 + 8 * s);
+                for (int k = 0; k < BK / 16; ++k)
+                  umma_bf16(d, sw128_desc(sa + 32 * k), sw128_desc(sb + 32 * k), idesc,
+                            (kb > 0 || k > 0) ? 1u : 0u);
+                umma_commit(empty0 + 8 * s);
+              }
+              __syncwarp();
             }
-            umma_commit(acc0 + 8 * t);
+            if (elect_one()) umma_commit(acc0 + 8 * t);
+            __syncwarp();
           }
     }
   } else {
-    const int q = warp & 3, half = warp >> 2;
+    const int q = warp & 3, part = warp >> 2;
     const int r = q * 32 + lane;
     uint32_t acc_ph[kPair] = {0, 0};
-    // the ReLU mask words of this thread's row and column half, one step
+    // the ReLU mask words of this thread's row and columns, one step
     // ahead: a tile's next layer is loaded while this one is processed
-    uint4 nb[kPair];
-    auto load_bits = [&](int layer, int m) {
-      return m < a.Mp ? __ldg(reinterpret_cast<const uint4*>(
-                                  a.bits + ((size_t)layer * a.Mp + m) * (kW / 32)) +
-                              half)
-                      : make_uint4(0u, 0u, 0u, 0u);
+    struct Bits {
+      uint2 k[kBlocks];
+    };
+    Bits nb[kPair];
+    auto load_bits = [&](int layer, int tile) {
+      Bits v;
+#pragma unroll
+      for (int k = 0; k < kBlocks; ++k)
+        v.k[k] = tile < a.n_tiles
+                     ? __ldg(reinterpret_cast<const uint2*>(a.bits + (size_t)layer * a.Mp * (kW / 32) +
+                                                            mask_at(tile, q, part * kBlocks + k, lane)))
+                     : make_uint2(0u, 0u);
+      return v;
     };
     bool ok = true;
     for (int pr = blockIdx.x; ok && pr < n_pairs; pr += gridDim.x) {
@@ -1068,15 +1315,19 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
       for (int t = 0; t < kPair; ++t) {
         // step 0's operand: BF16 dL/d(delta) in columns 0..2 of k-block 0
         const int m = (pr * kPair + t) * BM + r;
-        nb[t] = load_bits(kDepth - 1, m);
-        float v[32];
+        nb[t] = load_bits(kDepth - 1, pr * kPair + t);
+        float v[16];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = 0.f;
-        if (half == 0 && m < a.M)
-          for (int j = 0; j < 3; ++j) v[j] = a.dd[(size_t)m * 3 + j];
-        store_act32(smem + t * kActBytes, r, 32 * half, v);  // (free: waited at step 8)
+        for (int j = 0; j < 16; ++j) v[j] = 0.f;
+        for (int c = 64 - 16; c > 0; c -= 16)  // (free: waited at step 8)
+          if ((c >> 4) % kParts == part) store_act16(smem + t * kActBytes, r, c, v);
+        if (part == 0) {
+          if (m < a.M)
+            for (int j = 0; j < 3; ++j) v[j] = a.dd[(size_t)m * 3 + j];
+          store_act16(smem + t * kActBytes, r, 0, v);
+        }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("bar.sync 1, 256;" ::: "memory");
+        epi_sync();
         if (threadIdx.x == 0) mbar_arrive(actr0 + 8 * t);
       }
       for (int st = 0; ok && st < kSteps; ++st)
@@ -1086,34 +1337,37 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
             *s_ok = mbar_wait(acc0 + 8 * t, acc_ph[t], status, wait_ns) ? 1 : 0;
           // the tile's last store has read it before it is written again
           if (threadIdx.x == 32 * t) bulk_wait_read();
-          asm volatile("bar.sync 1, 256;" ::: "memory");
+          epi_sync();
           if (!(ok = *s_ok != 0)) break;  // (rewritten only after the step's last barrier)
           acc_ph[t] ^= 1u;
           tc_fence_after();
           const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(t * kW);
-          const int m = (pr * kPair + t) * BM + r;
           if (st < kDepth) {
             const int j = kDepth - 1 - st;  // the layer whose dZ this step forms
-            uint8_t* act = smem + t * kActBytes;
-            const uint4 mk = nb[t];
-            if (j > 0) nb[t] = load_bits(j - 1, m);
-#pragma unroll 1
-            for (int h2 = 0; h2 < 2; ++h2) {
-              const int c0 = half * (kW / 2) + 64 * h2;
-              const uint32_t mk0 = h2 ? mk.z : mk.x, mk1 = h2 ? mk.w : mk.y;
-              float vv[64];
-              tmem_ld64(trow + (uint32_t)c0, vv);
+            const FragStore fs = frag_store(act_s + t * kActBytes, q, lane);
+            const Bits mk = nb[t];
+            if (j > 0) nb[t] = load_bits(j - 1, pr * kPair + t);
 #pragma unroll
-              for (int k = 0; k < 32; ++k) {
-                if (!((mk0 >> k) & 1u)) vv[k] = 0.f;
-                if (!((mk1 >> k) & 1u)) vv[32 + k] = 0.f;
-              }
-              store_act32(act, r, c0, vv);
-              store_act32(act, r, c0 + 32, vv + 32);
+            for (int k = 0; k < kBlocks; ++k) {
+              const int cb = part * kBlocks + k;
+              float v[64];
+              tmem_ld64_frag(trow + (uint32_t)(cb * 64), v);
+              tmem_wait_ld();
+#pragma unroll
+              for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int g = 0; g < 8; g += 2) {
+                  const uint32_t bits = h ? mk.k[k].y : mk.k[k].x;
+                  const float* e = v + 32 * h + 4 * g;
+                  store_frag(fs, cb, h, g, pack_bf16(e[0], e[1]) & mask_pair<0>(bits, g),
+                             pack_bf16(e[2], e[3]) & mask_pair<1>(bits, g),
+                             pack_bf16(e[4], e[5]) & mask_pair<0>(bits, g + 1),
+                             pack_bf16(e[6], e[7]) & mask_pair<1>(bits, g + 1));
+                }
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             tc_fence_before();
-            asm volatile("bar.sync 1, 256;" ::: "memory");
+            epi_sync();
             if (threadIdx.x == 0) mbar_arrive(actr0 + 8 * t);
             if (threadIdx.x == 32 * t && pr * kPair + t < a.n_tiles) {
               for (int kb = 0; kb < kW / BK; ++kb)
@@ -1122,21 +1376,26 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
               bulk_commit();
             }
           } else {
-            if (half == 0) {
 #pragma unroll 1
-              for (int c = 0; c < kIn; c += 32) {
-                float v[32];
-                tmem_ld32(trow + (uint32_t)c, v);
-                if (m < a.Mp) {
-                  float4* d = reinterpret_cast<float4*>(a.denc + (size_t)m * kIn + c);
+            for (int cb = part; cb < kIn / 64; cb += kParts) {
+              float v[64];
+              tmem_ld64_frag(trow + (uint32_t)(cb * 64), v);
+              tmem_wait_ld();
+              if (pr * kPair + t < a.n_tiles) {
+                float* d = a.denc + ((size_t)(pr * kPair + t) * BM + q * 32 + (lane >> 2)) * kIn +
+                           cb * 64 + 2 * (lane & 3);
 #pragma unroll
-                  for (int k = 0; k < 8; ++k)
-                    d[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
-                }
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                  for (int g = 0; g < 8; ++g)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+                      *reinterpret_cast<float2*>(d + (16 * h + 8 * i) * kIn + 8 * g) =
+                          make_float2(v[32 * h + 4 * g + 2 * i], v[32 * h + 4 * g + 2 * i + 1]);
               }
             }
             tc_fence_before();
-            asm volatile("bar.sync 1, 256;" ::: "memory");  // TMEM drained before the next pair
+            epi_sync();  // TMEM drained before the next pair
           }
         }
     }
@@ -1448,13 +1707,15 @@ extern "C" gftorf_status gftorf_mlp_backward(int32_t n_gaussians, int32_t n_fram
   auto ldb_of = [&](int l) { return (l == 0 ? kIn : kW) + kExt; };
   const bool inj_loads = g_inject.load(std::memory_order_relaxed) == 1;
   const unsigned long long wait_ns = inj_loads ? 50000000ull : 2000000000ull;
-  mlp_head_grad_kernel<<<(Mp + 127) / 128, 128, 0, st>>>(d_delta, L.M, Mp, dzh, dzht,
-                                                         dbias_of(kDepth), kW + kExt);
+  const bool layerwise = g_inject.load(std::memory_order_relaxed) == 2;
+  mlp_head_grad_kernel<<<min((Mp + kHeadGradThreads - 1) / kHeadGradThreads, 4 * sms),
+                         kHeadGradThreads, 0, st>>>(d_delta, L.M, Mp, layerwise ? dzh : nullptr,
+                                                    dzht, dbias_of(kDepth), kW + kExt);
   count_launches(1);
   // head: dW_head += dZh^T H_7 (H_7 read MN-major)
   {
     CUtensorMap ma, mb;
-    if (!make_map(&ma, dzht, kHeadRows, Mp, Mp, BM) ||
+    if (!make_map(&ma, dzht, 3, Mp, Mp, BM) ||
         !make_map(&mb, H(kDepth - 1), Mp, kW, kW, BK))
       return GFTORF_ERR_CUDA;
     GemmArgs a;
@@ -1465,7 +1726,7 @@ extern "C" gftorf_status gftorf_mlp_backward(int32_t n_gaussians, int32_t n_fram
     a.status = status, a.inject_no_loads = inj_loads, a.wait_ns = wait_ns;
     if (!gemm<256, EPI_ATOMIC, 1, 0, 1>(ma, mb, a, 1, 1, splits, st)) return GFTORF_ERR_CUDA;
   }
-  if (g_inject.load(std::memory_order_relaxed) != 2) {
+  if (!layerwise) {
     // fused dZ chain: all layers per pair of 128-row tiles, dZ_l kept in
     // shared memory as the next layer's operand and stored (row-major) for
     // the weight gradients below
@@ -1532,12 +1793,12 @@ extern "C" gftorf_status gftorf_mlp_backward(int32_t n_gaussians, int32_t n_fram
     if (!(l == 0 ? gemm<kIn, EPI_PARTIAL, 2, 1, 1>(ma, mb, a, 1, 1, splits, st)
                  : gemm<kW, EPI_PARTIAL, 2, 1, 1>(ma, mb, a, 1, 1, splits, st)))
       return GFTORF_ERR_CUDA;
-    mlp_reduce_dw_kernel<<<(kW * K + 255) / 256, 256, 0, st>>>(part, splits, K, dwx + dwx_off(l),
+    mlp_reduce_dw_kernel<<<kW * K / 128, 32 * kReduceWarps, 0, st>>>(part, splits, K, dwx + dwx_off(l),
                                                                K + kExt);
     count_launches(1);
   }
   mlp_unpack_grads_kernel<<<4 * 152, 256, 0, st>>>(dwx, d_theta);
-  mlp_encode_bwd_kernel<<<(n_gaussians + 7) / 8, 256, 0, st>>>(means, denc, n_gaussians,
+  mlp_encode_bwd_kernel<<<(n_gaussians + 63) / 64, 128, 0, st>>>(means, denc, n_gaussians,
                                                                n_frames, inv_scale, d_means);
   count_launches(2);
   (void)times;
