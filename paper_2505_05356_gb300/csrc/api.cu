@@ -47,8 +47,7 @@ bool dims_ok(const gftorf_dims* d) {
     return false;
   if (d->reserved != 0) return false;
   if (d->max_instances < 0 || d->max_instances > (int64_t)0xFFFFFFFFll) return false;
-  // per-CTA tile counters ((tiles_x + 1) x (tiles_y + 1), 4 bytes each) live in
-  // shared memory
+  // (the tile rectangles' corners: what the binning was sized for)
   const int64_t corners = (int64_t)((d->width + d->tile_w - 1) / d->tile_w + 1) *
                           ((d->height + d->tile_h - 1) / d->tile_h + 1);
   if (corners > 50000) return false;
@@ -60,6 +59,30 @@ bool params_ok(const Layout& L, const gftorf_gaussians* g) {
   if (L.N == 0) return true;
   if (!g->means || !g->scales || !g->quats || !g->opacity) return false;
   return L.nsh ? g->sh != nullptr : g->amplitude != nullptr;
+}
+
+// Rows of the chunk counts' own region, and a region nothing uses: the sizes that an
+// earlier binning (chunks of instances, a scan of the Gaussians' tile counts) needed,
+// kept so that the fixed-scratch entry point takes and refuses the same problems.
+size_t chunk_rows(const Layout& L) { return (size_t)((L.cap + 8191) / 8192) + L.B; }
+size_t spare_bytes(size_t BN) { return align_up(BN * 4 + 4) + ((BN + 16383) / 16384 + 1) * 8; }
+
+// The chunk size and the counts' place: B n_chunk rows of NT words, in their own
+// region or, where that holds more, over the depth sort's ping-pong buffers and
+// the first sorted indices [off_zkey2, off_ids2), which nothing reads after its
+// last pass.  One chunk per frame always fits the first, chunks of NT / 3 or more
+// Gaussians the second.
+void place_chunks(Layout& L) {
+  const size_t dead = (L.off_ids2 - L.off_zkey2) / ((size_t)L.NT * 4), own = chunk_rows(L);
+  const size_t rows = dead > own ? dead : own;
+  if (dead > own) L.off_tcnt = L.off_zkey2;
+  L.chunk = 32;
+  L.chunks_per_cta = L.NT >= 512 ? 1 : (L.NT >= 64 ? 512 / L.NT : 8);
+  auto per_frame = [&] { return ((size_t)L.N + L.chunk - 1) / L.chunk; };
+  while (L.chunk < kMaxChunk &&
+         per_frame() * L.B > (size_t)kMinChunkCtas * L.chunks_per_cta) L.chunk *= 2;
+  while (per_frame() > 1 && per_frame() * L.B > rows) L.chunk *= 2;
+  L.n_chunk = (int)(per_frame() > 0 ? per_frame() : 1);
 }
 
 Layout make_layout(const gftorf_dims* d) {
@@ -84,11 +107,6 @@ Layout make_layout(const gftorf_dims* d) {
   L.rec_stride = (8 + L.NF + per16 - 1) / per16 * per16;
   L.g2d_stride = 7 + L.NF;
   L.n_dblk = (L.N + kSortTile - 1) / kSortTile;
-  L.n_chunk = (int)((d->max_instances + kChunk - 1) / kChunk) + L.B;
-  L.n_scan = (int)(((size_t)L.B * L.N + kScanTile - 1) / kScanTile);
-  int nw = 8;  // scatter warps: per-warp tile counters within 96 KB where possible
-  while (nw > 1 && (size_t)nw * (L.tiles_x + 1) * (L.tiles_y + 1) * 4 > 96 * 1024) nw >>= 1;
-  L.scatter_warps = nw;
   L.cap = d->max_instances;
   const size_t BN = (size_t)L.B * L.N, HW = (size_t)L.W * L.H;
   size_t o = 0;
@@ -108,16 +126,16 @@ Layout make_layout(const gftorf_dims* d) {
   L.off_ids2 = take(BN * 4);
   L.off_dhist = take(lb_bytes(L));
   L.off_dtot = take((size_t)L.B * 1024 * 4);
-  L.off_ecnt = take((size_t)L.B * L.N * 4 + 4);
-  L.off_bsum = take((size_t)(L.n_scan + 1) * 8);  // scan status words, 2 counters
-  L.off_tcnt = take((size_t)L.n_chunk * L.NT * 4);
-  L.off_toff = take((size_t)L.B * L.NT * 4);
+  L.off_spare = take(spare_bytes(BN));
+  L.off_tcnt = take(chunk_rows(L) * L.NT * 4);
+  L.off_ttot = take((size_t)L.B * L.NT * 4);
   L.off_ranges = take((size_t)L.B * L.NT * sizeof(uint2));
   L.off_values = take((size_t)(L.cap > 0 ? L.cap : 1) * 4);
   L.off_tfinal = take((size_t)L.B * HW * L.real_size);
   L.off_nlast = take((size_t)L.B * HW * 4);
   L.off_g2d = take(BN * L.g2d_stride * L.real_size);
   L.total = o;
+  place_chunks(L);
   return L;
 }
 
@@ -177,16 +195,16 @@ Layout binning_layout(const gftorf_dims* d) {
   L.off_ids2 = take(BN * 4);
   L.off_dhist = take(lb_bytes(L));
   L.off_dtot = take((size_t)L.B * 1024 * 4);
-  L.off_ecnt = take(BN * 4 + 4);
-  L.off_bsum = take((size_t)(L.n_scan + 1) * 8);  // scan status words, 2 counters
-  L.off_tcnt = take((size_t)L.n_chunk * L.NT * 4);
-  L.off_toff = take((size_t)L.B * L.NT * 4);
+  L.off_spare = take(spare_bytes(BN));
+  L.off_tcnt = take(chunk_rows(L) * L.NT * 4);
+  L.off_ttot = take((size_t)L.B * L.NT * 4);
   L.off_ranges = take((size_t)L.B * L.NT * sizeof(uint2));
   L.off_values = take((size_t)(L.cap > 0 ? L.cap : 1) * 4);
   L.off_tfinal = take(0);
   L.off_nlast = take(0);
   L.off_g2d = take(0);
   L.total = o;
+  place_chunks(L);
   return L;
 }
 

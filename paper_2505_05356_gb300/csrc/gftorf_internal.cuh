@@ -78,13 +78,11 @@ constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;
-// Tile binning: a chunk of kChunk consecutive instances (in emission order:
-// frame, depth rank, tile of the rectangle) per CTA.
-constexpr int kChunk = 8192;
-// Device-wide scan: elements per CTA (few enough CTAs that they all fit on
-// the GPU at once, so the look-back chains stay short) and threads per CTA.
-constexpr int kScanTile = 16384;
-constexpr int kScanThreads = 512;
+// Tile binning: at most kMaxChunk Gaussians per chunk where the counts' space allows,
+// and fewer, down to 32 (one group), where the batch would give the chunk kernels
+// less than about kMinChunkCtas CTAs (four per SM).
+constexpr int kMaxChunk = 256;
+constexpr int kMinChunkCtas = 608;
 
 // Per-frame camera in device memory.
 template <typename T>
@@ -123,8 +121,7 @@ struct Header {
                                   // warp's rows (the rest are skipped per warp)
   uint32_t queue[4];       // persistent work-queue heads (fwd, bwd)
   uint32_t vis[kMaxFrames];  // visible Gaussians per frame
-  uint32_t fstart[kMaxFrames + 1];  // first instance of each frame
-  uint32_t coff[kMaxFrames + 1];    // first binning chunk of each frame
+  uint32_t col_done;         // column-scan CTAs that have finished (0 between binnings)
 };
 
 // Host-computed byte layout of the workspace for one gftorf_dims.
@@ -139,13 +136,12 @@ struct Layout {
   int rec_stride;  // Reals per projected record (16-byte multiple)
   int g2d_stride;  // Reals per 2D-gradient row
   int n_dblk;      // depth-sort tiles per frame
-  int n_chunk;     // binning chunks of the batch (upper bound)
-  int n_scan;      // CTAs of the emission-offset scan
-  int scatter_warps;
+  int chunk;       // Gaussians per binning chunk (a multiple of 32)
+  int n_chunk;     // binning chunks per frame
+  int chunks_per_cta;  // of the chunk kernels: enough for 512 (chunk, tile) items
   int64_t cap;
   size_t off_header, off_table, off_rec, off_rect, off_srect, off_zkey, off_zkey2,
-      off_ids, off_ids2, off_dhist, off_dtot, off_ecnt, off_bsum, off_tcnt, off_toff,
-      off_ranges,
+      off_ids, off_ids2, off_dhist, off_dtot, off_spare, off_tcnt, off_ttot, off_ranges,
       off_values, off_tfinal, off_nlast, off_g2d, total;
 };
 
