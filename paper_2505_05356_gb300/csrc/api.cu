@@ -61,6 +61,19 @@ bool params_ok(const Layout& L, const gftorf_gaussians* g) {
   return L.nsh ? g->sh != nullptr : g->amplitude != nullptr;
 }
 
+// Pixels per thread where the caller leaves the choice (the results do not depend on
+// it): 4 shares most of a record's work, 1 gives the most warps.  With about 24
+// resident warps on 152 SMs, one pixel per thread as long as all warps are resident
+// at once (3 frames of 96x64 pixels, fwd+bwd: 217 us with 2, 181 with 1), four where
+// they fill the GPU several times over (12 frames of 517x389, forward: 639 us with
+// 2, 622 with 4), else two.  Tiles 32 wide or more have four.
+int default_ppt(const Layout& L) {
+  if (L.TW >= 32) return 4;
+  const int64_t resident = 152 * 24, warps1 = (int64_t)L.B * L.NT * (L.TW * L.TH / 32);
+  if (warps1 <= resident) return 1;
+  return warps1 >= 16 * resident && L.TW * L.TH / 4 >= 32 ? 4 : 2;
+}
+
 // Rows of the chunk counts' own region, and a region nothing uses: the sizes that an
 // earlier binning (chunks of instances, a scan of the Gaussians' tile counts) needed,
 // kept so that the fixed-scratch entry point takes and refuses the same problems.
@@ -93,7 +106,7 @@ Layout make_layout(const gftorf_dims* d) {
   L.C = L.F * L.P + 1, L.NF = 2 * L.F + 1, L.dtype = d->dtype;
   L.real_size = d->dtype == GFTORF_F64 ? 8 : 4;
   L.mode = d->render_mode;
-  L.ppt = d->pixels_per_thread ? d->pixels_per_thread : (d->tile_w >= 32 ? 4 : 2);
+  L.ppt = d->pixels_per_thread;
   L.cull = (d->flags & GFTORF_FLAG_NO_TILE_CULL) ? 0 : 1;
   L.count_pairs = (d->flags & GFTORF_FLAG_COUNT_PAIRS) ? 1 : 0;
   L.phasor = (d->flags & GFTORF_FLAG_PHASOR) ? 1 : 0;
@@ -103,6 +116,7 @@ Layout make_layout(const gftorf_dims* d) {
   L.tiles_x = (L.W + L.TW - 1) / L.TW;
   L.tiles_y = (L.H + L.TH - 1) / L.TH;
   L.NT = L.tiles_x * L.tiles_y;
+  if (L.ppt == 0) L.ppt = default_ppt(L);
   const int per16 = 16 / L.real_size;
   L.rec_stride = (8 + L.NF + per16 - 1) / per16 * per16;
   L.g2d_stride = 7 + L.NF;
@@ -151,8 +165,11 @@ gftorf_status launch_status() {
 }
 
 // Writes the batch table into the workspace from a kernel argument, so the
-// upload is an ordinary kernel node inside a captured graph.
-__global__ void store_table_kernel(Table t, Table* dst) {
+// upload is an ordinary kernel node inside a captured graph; clears the header too.
+__global__ void store_table_kernel(Table t, Table* dst, Header* hdr) {
+  grid_begin_early();
+  for (int i = threadIdx.x; i < (int)(sizeof(Header) / 4); i += blockDim.x)
+    reinterpret_cast<uint32_t*>(hdr)[i] = 0u;
   const int n = sizeof(Table) / sizeof(double);
   const double* s = reinterpret_cast<const double*>(&t);
   double* d = reinterpret_cast<double*>(dst);
@@ -320,8 +337,8 @@ gftorf_status gftorf_preprocess(const gftorf_dims* dims,
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   unsigned char* ws = static_cast<unsigned char*>(workspace);
-  cudaMemsetAsync(ws + L.off_header, 0, sizeof(Header), st);
-  store_table_kernel<<<1, 256, 0, st>>>(t, at<Table>(ws, L.off_table));
+  launch(store_table_kernel, 1, 256, 0, st, t, at<Table>(ws, L.off_table),
+         at<Header>(ws, L.off_header));
   count_launches(1);
   if (L.dtype == GFTORF_F32)
     launch_preprocess<float>(L, *g, ws, st);

@@ -120,6 +120,7 @@ __global__ void footprint_kernel(const float* __restrict__ u,
                                  uint2* __restrict__ rect,
                                  uint32_t* __restrict__ zkey, int N, int TW,
                                  int TH, int tiles_x, int tiles_y) {
+  grid_begin_early();
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   const int b = blockIdx.y;
   bool visible = false;
@@ -163,6 +164,7 @@ constexpr int kLbSpinLimit = 1 << 22;  // bounded wait on a predecessor tile
 
 __global__ void __launch_bounds__(kSortThreads)
     dsort_hist_kernel(const uint32_t* __restrict__ keys, int N, uint32_t* __restrict__ ghist) {
+  grid_begin_early();
   __shared__ uint32_t h[4][256];
   const int blk = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
   for (int i = tid; i < 4 * 256; i += kSortThreads) (&h[0][0])[i] = 0;
@@ -188,6 +190,7 @@ __global__ void __launch_bounds__(kSortThreads)
 
 // per (frame, pass): exclusive scan of the 256 digit totals -> digit bases
 __global__ void __launch_bounds__(256) dsort_bases_kernel(uint32_t* __restrict__ ghist) {
+  grid_begin_early();
   cta_exclusive_scan<uint32_t>(ghist + (size_t)blockIdx.x * 256, 256, nullptr);
 }
 
@@ -202,6 +205,7 @@ __global__ void __launch_bounds__(kSortThreads, 5)  // <= 48 registers, no spill
                       uint32_t* __restrict__ status, uint32_t* __restrict__ tile_counter,
                       Header* __restrict__ hdr, const uint2* __restrict__ rin,
                       uint2* __restrict__ rout) {
+  grid_begin_early();
   __shared__ uint32_t wc[kSortWarps][256];
   __shared__ uint32_t s_tile;
   // the tile's keys and indices in digit order (staged, then written out in
@@ -418,6 +422,7 @@ constexpr int kBinThreads = 256;
 __global__ void __launch_bounds__(kBinThreads)
     tile_count_kernel(const uint2* __restrict__ srect, const Header* __restrict__ hdr,
                       uint32_t* __restrict__ tcnt, ChunkArgs a) {
+  grid_begin_early();
   extern __shared__ uint32_t smem[];
   const int b = blockIdx.y, c0 = blockIdx.x * a.per_cta, vis = (int)hdr->vis[b];
   const int r0 = c0 * a.chunk, r1 = min(r0 + a.per_cta * a.chunk, vis);
@@ -456,6 +461,7 @@ __global__ void __launch_bounds__(32 * kColWarps)
     tile_colscan_kernel(uint32_t* __restrict__ tcnt, uint32_t* __restrict__ ttot,
                         uint2* __restrict__ ranges, Header* __restrict__ hdr, ChunkArgs a,
                         int64_t cap) {
+  grid_begin_early();
   __shared__ uint32_t s_seg[kColWarps][32];
   __shared__ uint64_t s_w[kColWarps];
   __shared__ bool s_last;
@@ -538,6 +544,7 @@ __global__ void __launch_bounds__(kBinThreads)
                         const Header* __restrict__ hdr, uint32_t* __restrict__ tcnt,
                         const uint2* __restrict__ ranges, uint32_t* __restrict__ values,
                         ChunkArgs a, int64_t cap) {
+  grid_begin();
   extern __shared__ uint32_t smem[];
   const int b = blockIdx.y, c0 = blockIdx.x * a.per_cta, vis = (int)hdr->vis[b];
   const int r0 = c0 * a.chunk, r1 = min(r0 + a.per_cta * a.chunk, vis);
@@ -595,6 +602,7 @@ __global__ void export_keys_kernel(const uint2* __restrict__ ranges,
                                    const uint32_t* __restrict__ values,
                                    const uint32_t* __restrict__ zkey,
                                    uint64_t* __restrict__ keys, int N, int NT) {
+  grid_begin();
   const int t = blockIdx.x, b = blockIdx.y;
   const uint2 r = ranges[(size_t)b * NT + t];
   const uint64_t hi = ((uint64_t)b * NT + t) << 32;
@@ -617,7 +625,7 @@ void launch_footprints(const Layout& L, const float* u, const float* v,
                        unsigned char* ws, cudaStream_t st) {
   if (L.N == 0) return;
   dim3 grid((L.N + 255) / 256, L.B);
-  footprint_kernel<<<grid, 256, 0, st>>>(
+  launch(footprint_kernel, grid, 256, 0, st,
       u, v, radius, z, at<Header>(ws, L.off_header), at<uint2>(ws, L.off_rect),
       at<uint32_t>(ws, L.off_zkey), L.N, L.TW, L.TH, L.tiles_x, L.tiles_y);
   count_launches(1);
@@ -651,10 +659,10 @@ void launch_binning(const Layout& L, unsigned char* ws, cudaStream_t st) {
   uint32_t* iout[2] = {i0, i1};
   // the look-back words and the digit totals are adjacent: one memset
   cudaMemsetAsync(lb, 0, L.off_dtot + (size_t)L.B * 1024 * 4 - L.off_dhist, st);
-  dsort_hist_kernel<<<dim3(L.n_dblk, L.B), kSortThreads, 0, st>>>(zkey, L.N, ghist);
-  dsort_bases_kernel<<<L.B * 4, 256, 0, st>>>(ghist);
+  launch(dsort_hist_kernel, dim3(L.n_dblk, L.B), kSortThreads, 0, st, zkey, L.N, ghist);
+  launch(dsort_bases_kernel, L.B * 4, 256, 0, st, ghist);
   for (int pass = 0; pass < 4; ++pass) {
-    dsort_pass_kernel<<<L.B * L.n_dblk, kSortThreads, 0, st>>>(
+    launch(dsort_pass_kernel, L.B * L.n_dblk, kSortThreads, 0, st,
         kin, iin, kout[pass & 1], iout[pass & 1], L.N, L.B, pass, L.n_dblk, ghist,
         lb + kLbCounters, lb + pass, hdr, pass == 3 ? rect : nullptr,
         pass == 3 ? srect : nullptr);
@@ -668,11 +676,13 @@ void launch_binning(const Layout& L, unsigned char* ws, cudaStream_t st) {
   const ChunkArgs a{L.N, L.NT, L.tiles_x, L.tiles_y, L.chunk, L.n_chunk, L.chunks_per_cta, piece};
   const dim3 ctas((L.n_chunk + L.chunks_per_cta - 1) / L.chunks_per_cta, L.B);
   const size_t smem = (size_t)piece * stride * 4;
-  tile_count_kernel<<<ctas, kBinThreads, smem, st>>>(srect, hdr, tcnt, a);
-  tile_colscan_kernel<<<dim3((L.NT + 31) / 32, L.B), 32 * kColWarps, 0, st>>>(tcnt, ttot, ranges,
+  launch(tile_count_kernel, ctas, kBinThreads, smem, st, srect, hdr, tcnt, a);
+  launch(tile_colscan_kernel, dim3((L.NT + 31) / 32, L.B), 32 * kColWarps, 0, st,
+         tcnt, ttot, ranges,
                                                                               hdr, a, L.cap);
   // 4. stable scatter
-  tile_scatter_kernel<<<ctas, kBinThreads, smem, st>>>(sorted, srect, hdr, tcnt, ranges, values, a,
+  launch(tile_scatter_kernel, ctas, kBinThreads, smem, st,
+         sorted, srect, hdr, tcnt, ranges, values, a,
                                                        L.cap);
   count_launches(9);
 }
@@ -680,7 +690,7 @@ void launch_binning(const Layout& L, unsigned char* ws, cudaStream_t st) {
 void launch_export_keys(const Layout& L, uint64_t* keys, unsigned char* ws,
                         cudaStream_t st) {
   dim3 g(L.NT, L.B);
-  export_keys_kernel<<<g, 128, 0, st>>>(
+  launch(export_keys_kernel, g, 128, 0, st,
       at<const uint2>(ws, L.off_ranges), at<const uint32_t>(ws, L.off_values),
       at<const uint32_t>(ws, L.off_zkey), keys, L.N, L.NT);
   count_launches(1);

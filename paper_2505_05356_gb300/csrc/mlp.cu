@@ -405,6 +405,7 @@ template <int BN, int EPI, int MT, int MNA, int MNB>
 __global__ void __launch_bounds__(192, MT == 2 ? 1 : 2)
     umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
                      const __grid_constant__ CUtensorMap tmB, const GemmArgs p) {
+  grid_begin();
   using S = GemmShape<BN, MT>;
   constexpr int kStages = S::kStages, A_BYTES = S::A_BYTES, STAGE = S::STAGE;
   constexpr uint32_t TCOLS = S::TCOLS;
@@ -574,6 +575,7 @@ __host__ __device__ constexpr size_t head_bias_off_dev() {
 __global__ void mlp_prep_weights_kernel(const float* __restrict__ theta,
                                         __nv_bfloat16* __restrict__ wb,
                                         __nv_bfloat16* __restrict__ wt) {
+  grid_begin_early();
   // packed offsets: layer l (0..7) W at off_w(l), then b; head after
   const int K0 = kIn;
   const size_t total = (size_t)kW * K0 + (size_t)(kDepth - 1) * kW * kW + (size_t)kHeadRows * kW;
@@ -640,6 +642,7 @@ __device__ __forceinline__ void encode_row(const float* __restrict__ means, cons
 // positional encoding of row m = b N + g into enc[m][0..127]
 __global__ void mlp_encode_kernel(const float* __restrict__ means, Times tm, int N, int B,
                                   float inv_scale, int M_pad, __nv_bfloat16* __restrict__ enc) {
+  grid_begin();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= M_pad) return;
   float e[kIn];
@@ -660,6 +663,7 @@ __global__ void __launch_bounds__(kHeadGradThreads)
     mlp_head_grad_kernel(const float* __restrict__ dd, int M, int M_pad,
                          __nv_bfloat16* __restrict__ dz, __nv_bfloat16* __restrict__ dzt,
                          float* __restrict__ dbias, int ldb) {
+  grid_begin_early();
   __shared__ float s_sum[kHeadGradThreads / 32][3];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float sum[3] = {0.f, 0.f, 0.f};
@@ -703,6 +707,7 @@ __global__ void __launch_bounds__(kHeadGradThreads)
 __global__ void __launch_bounds__(128)
     mlp_encode_bwd_kernel(const float* __restrict__ means, const float* __restrict__ denc, int N,
                           int B, float inv_scale, float* __restrict__ dmeans) {
+  grid_begin();
   constexpr int kBands = kFreq / 2, kCols = 6 * kBands + 4;  // (even: float2 loads)
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int g = min(i >> 1, N - 1), h = i & 1;  // (a whole warp reaches the shuffles)
@@ -744,6 +749,7 @@ __global__ void __launch_bounds__(128)
 
 // extended weight gradients [rows][K + ext] -> packed d_theta (W then b)
 __global__ void mlp_unpack_grads_kernel(const float* __restrict__ dwx, float* __restrict__ dth) {
+  grid_begin_early();
   const size_t total = (size_t)kW * (kIn + 1) + (size_t)(kDepth - 1) * kW * (kW + 1) + 3 * (kW + 1);
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
        e += (size_t)gridDim.x * blockDim.x) {
@@ -780,6 +786,7 @@ constexpr int kReduceWarps = 8;
 __global__ void __launch_bounds__(32 * kReduceWarps)
     mlp_reduce_dw_kernel(const float* __restrict__ part, int splits, int K,
                          float* __restrict__ dw, int ld) {
+  grid_begin_early();
   __shared__ float4 s_sum[kReduceWarps][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int e = (blockIdx.x * 32 + lane) * 4;  // 256 K is a multiple of 128
@@ -978,6 +985,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
                          const float* __restrict__ means, Times tm, int N, int M, int n_tiles,
                          float inv_scale, float* __restrict__ delta, int* status,
                          unsigned long long wait_ns, int inject_no_loads, FusedKeep keep) {
+  grid_begin();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem =
       reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -1200,6 +1208,7 @@ struct FusedBwdArgs {
 __global__ void __launch_bounds__(kFusedThreads, 1)
     mlp_fused_bwd_kernel(const __grid_constant__ FusedMaps maps, const FusedBwdArgs a,
                          int* status, unsigned long long wait_ns, int inject_no_loads) {
+  grid_begin();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem =
       reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -1450,8 +1459,8 @@ bool gemm(const CUtensorMap& a, const CUtensorMap& b, const GemmArgs& args, int 
                                     smem) == cudaSuccess;
       }))
     return false;
-  umma_gemm_kernel<BN, EPI, MT, MNA, MNB>
-      <<<dim3(m_tiles, n_tiles, splits), 192, smem, st>>>(a, b, args);
+  launch(umma_gemm_kernel<BN, EPI, MT, MNA, MNB>, dim3(m_tiles, n_tiles, splits), 192, smem, st,
+         a, b, args);
   count_launches(1);
   return true;
 }
@@ -1590,7 +1599,7 @@ extern "C" gftorf_status gftorf_mlp_forward(int32_t n_gaussians, int32_t n_frame
   if (L.M == 0) return cudaGetLastError() == cudaSuccess ? GFTORF_OK : GFTORF_ERR_CUDA;
   auto* wb = ptr<__nv_bfloat16>(ws, L.off_wb);
   auto* wt = ptr<__nv_bfloat16>(ws, L.off_wt);
-  mlp_prep_weights_kernel<<<4 * 152, 256, 0, st>>>(theta, wb, wt);
+  launch(mlp_prep_weights_kernel, 4 * 152, 256, 0, st, theta, wb, wt);
   Times tm;
   memset(&tm, 0, sizeof(tm));
   for (int b = 0; b < n_frames; ++b) tm.t[b] = times[b];
@@ -1614,13 +1623,13 @@ extern "C" gftorf_status gftorf_mlp_forward(int32_t n_gaussians, int32_t n_frame
     const int sms = sm_count();
     const int n_pairs = (mt + kPair - 1) / kPair;
     const int inj = g_inject.load();
-    mlp_fused_fwd_kernel<true><<<n_pairs < sms ? n_pairs : sms, kFusedThreads, kFusedSmem, st>>>(
+    launch(mlp_fused_fwd_kernel<true>, n_pairs < sms ? n_pairs : sms, kFusedThreads, kFusedSmem, st,
         maps, theta, means, tm, n_gaussians, L.M, mt, inv_scale, delta, status,
         inj == 1 ? 50000000ull : 2000000000ull, inj == 1, keep);
     count_launches(2);
     return cudaGetLastError() == cudaSuccess ? GFTORF_OK : GFTORF_ERR_CUDA;
   }
-  mlp_encode_kernel<<<(Mp + 127) / 128, 128, 0, st>>>(means, tm, n_gaussians, n_frames,
+  launch(mlp_encode_kernel, (Mp + 127) / 128, 128, 0, st, means, tm, n_gaussians, n_frames,
                                                       inv_scale, Mp, enc);
   count_launches(2);
   for (int l = 0; l < kDepth; ++l) {
@@ -1682,7 +1691,7 @@ extern "C" gftorf_status gftorf_mlp_backward(int32_t n_gaussians, int32_t n_fram
   float* dwx = ptr<float>(ws, L.off_dwx);
   cudaMemsetAsync(dwx, 0, dwx_floats() * 4, st);
   if (L.M == 0) {
-    mlp_unpack_grads_kernel<<<4 * 152, 256, 0, st>>>(dwx, d_theta);
+    launch(mlp_unpack_grads_kernel, 4 * 152, 256, 0, st, dwx, d_theta);
     count_launches(1);
     return cudaGetLastError() == cudaSuccess ? GFTORF_OK : GFTORF_ERR_CUDA;
   }
@@ -1708,8 +1717,9 @@ extern "C" gftorf_status gftorf_mlp_backward(int32_t n_gaussians, int32_t n_fram
   const bool inj_loads = g_inject.load(std::memory_order_relaxed) == 1;
   const unsigned long long wait_ns = inj_loads ? 50000000ull : 2000000000ull;
   const bool layerwise = g_inject.load(std::memory_order_relaxed) == 2;
-  mlp_head_grad_kernel<<<min((Mp + kHeadGradThreads - 1) / kHeadGradThreads, 4 * sms),
-                         kHeadGradThreads, 0, st>>>(d_delta, L.M, Mp, layerwise ? dzh : nullptr,
+  launch(mlp_head_grad_kernel, min((Mp + kHeadGradThreads - 1) / kHeadGradThreads, 4 * sms),
+         kHeadGradThreads, 0, st,
+         d_delta, L.M, Mp, layerwise ? dzh : nullptr,
                                                     dzht, dbias_of(kDepth), kW + kExt);
   count_launches(1);
   // head: dW_head += dZh^T H_7 (H_7 read MN-major)
@@ -1743,7 +1753,7 @@ extern "C" gftorf_status gftorf_mlp_backward(int32_t n_gaussians, int32_t n_fram
     fa.dd = d_delta, fa.bits = bits, fa.denc = denc;
     fa.M = L.M, fa.Mp = Mp, fa.n_tiles = mt;
     const int n_pairs = (mt + kPair - 1) / kPair;
-    mlp_fused_bwd_kernel<<<n_pairs < sms ? n_pairs : sms, kFusedThreads, kBwdSmem, st>>>(
+    launch(mlp_fused_bwd_kernel, n_pairs < sms ? n_pairs : sms, kFusedThreads, kBwdSmem, st,
         maps, fa, status, wait_ns, inj_loads);
     count_launches(1);
   } else {
@@ -1793,12 +1803,13 @@ extern "C" gftorf_status gftorf_mlp_backward(int32_t n_gaussians, int32_t n_fram
     if (!(l == 0 ? gemm<kIn, EPI_PARTIAL, 2, 1, 1>(ma, mb, a, 1, 1, splits, st)
                  : gemm<kW, EPI_PARTIAL, 2, 1, 1>(ma, mb, a, 1, 1, splits, st)))
       return GFTORF_ERR_CUDA;
-    mlp_reduce_dw_kernel<<<kW * K / 128, 32 * kReduceWarps, 0, st>>>(part, splits, K, dwx + dwx_off(l),
+    launch(mlp_reduce_dw_kernel, kW * K / 128, 32 * kReduceWarps, 0, st,
+           part, splits, K, dwx + dwx_off(l),
                                                                K + kExt);
     count_launches(1);
   }
-  mlp_unpack_grads_kernel<<<4 * 152, 256, 0, st>>>(dwx, d_theta);
-  mlp_encode_bwd_kernel<<<(n_gaussians + 63) / 64, 128, 0, st>>>(means, denc, n_gaussians,
+  launch(mlp_unpack_grads_kernel, 4 * 152, 256, 0, st, dwx, d_theta);
+  launch(mlp_encode_bwd_kernel, (n_gaussians + 63) / 64, 128, 0, st, means, denc, n_gaussians,
                                                                n_frames, inv_scale, d_means);
   count_launches(2);
   (void)times;
@@ -1866,7 +1877,7 @@ extern "C" gftorf_status gftorf_mlp_infer(int32_t n_gaussians, int32_t n_frames,
   if (M == 0) return cudaGetLastError() == cudaSuccess ? GFTORF_OK : GFTORF_ERR_CUDA;
   auto* wb = ptr<__nv_bfloat16>(workspace, 256);
   auto* wt = wb + wb_elems();
-  mlp_prep_weights_kernel<<<4 * 152, 256, 0, st>>>(theta, wb, wt);
+  launch(mlp_prep_weights_kernel, 4 * 152, 256, 0, st, theta, wb, wt);
   FusedMaps maps;
   for (int l = 0; l <= kDepth; ++l) {
     const int K = l == 0 ? kIn : kW, rows = l == kDepth ? kHeadRows : kW;
@@ -1882,7 +1893,7 @@ extern "C" gftorf_status gftorf_mlp_infer(int32_t n_gaussians, int32_t n_frames,
   const unsigned long long wait_ns = g_inject.load() == 1 ? 50000000ull : 2000000000ull;
   FusedKeep none;
   memset(&none, 0, sizeof(none));
-  mlp_fused_fwd_kernel<false><<<n_pairs < sms ? n_pairs : sms, kFusedThreads, kFusedSmem, st>>>(
+  launch(mlp_fused_fwd_kernel<false>, n_pairs < sms ? n_pairs : sms, kFusedThreads, kFusedSmem, st,
       maps, theta, means, tm, n_gaussians, M, n_tiles, inv_scale, delta, status, wait_ns,
       g_inject.load() == 1, none);
   count_launches(2);

@@ -289,6 +289,7 @@ __global__ void __launch_bounds__(256)
                       uint2* __restrict__ rect, uint32_t* __restrict__ zkey,
                       int N, int TW, int TH, int tiles_x, int tiles_y,
                       int rec_stride, int cull, int nsh) {
+  grid_begin();
   constexpr int NF = 2 * F + 1;
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   const int b = blockIdx.y;
@@ -391,6 +392,7 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 8 ? 1 : (SH ? 3 : 4))
                           const uint2* __restrict__ rect,
                           const Real* __restrict__ g2d, int g2d_stride, int N,
                           int B, int nsh) {
+  grid_begin();
   constexpr int NF = 2 * F + 1;
   constexpr int NS = SH ? kMaxSh : 1;
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
@@ -640,11 +642,11 @@ void launch_preprocess(const Layout& L, const gftorf_gaussians& g,
   auto* zkey = at<uint32_t>(ws, L.off_zkey);
 #define GFTORF_PRE(FF)                                                         \
   if (L.nsh)                                                                   \
-    preprocess_kernel<Real, FF, true><<<grid, 256, 0, st>>>(                   \
+    launch(preprocess_kernel<Real, FF, true>, grid, 256, 0, st,                    \
         g, tab, hdr, rec, rect, zkey, L.N, L.TW, L.TH, L.tiles_x, L.tiles_y,   \
         L.rec_stride, L.cull, L.nsh);                                          \
   else                                                                         \
-    preprocess_kernel<Real, FF, false><<<grid, 256, 0, st>>>(                  \
+    launch(preprocess_kernel<Real, FF, false>, grid, 256, 0, st,                   \
         g, tab, hdr, rec, rect, zkey, L.N, L.TW, L.TH, L.tiles_x, L.tiles_y,   \
         L.rec_stride, L.cull, 0)
   switch (L.F) {
@@ -668,10 +670,10 @@ void launch_preprocess_bwd(const Layout& L, const gftorf_gaussians& g,
   auto* g2d = at<const Real>(ws, L.off_g2d);
 #define GFTORF_PREB(FF)                                                        \
   if (L.nsh)                                                                   \
-    preprocess_bwd_kernel<Real, FF, true><<<grid, 128, 0, st>>>(               \
+    launch(preprocess_bwd_kernel<Real, FF, true>, grid, 128, 0, st,                \
         g, gr, tab, rect, g2d, L.g2d_stride, L.N, L.B, L.nsh);                 \
   else                                                                         \
-    preprocess_bwd_kernel<Real, FF, false><<<grid, 128, 0, st>>>(              \
+    launch(preprocess_bwd_kernel<Real, FF, false>, grid, 128, 0, st,               \
         g, gr, tab, rect, g2d, L.g2d_stride, L.N, L.B, 0)
   switch (L.F) {
     case 1: GFTORF_PREB(1); break;

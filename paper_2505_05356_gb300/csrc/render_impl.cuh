@@ -590,6 +590,7 @@ __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
                       const Real* __restrict__ rec, const Real* __restrict__ bg,
                       Real* __restrict__ out, Real* __restrict__ tfinal,
                       uint32_t* __restrict__ nlast, int persistent) {
+  grid_begin();
   constexpr int RS = rec_stride<Real, F>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real* s_rec = reinterpret_cast<Real*>(smem_raw);
@@ -920,6 +921,7 @@ __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
                       const Real* __restrict__ tfinal,
                       const uint32_t* __restrict__ nlast, Real* __restrict__ g2d,
                       int g2d_stride, Real* __restrict__ dbg, int persistent) {
+  grid_begin();
   constexpr int NF = 2 * F + 1;
   constexpr int GS = 6 + NF + (DEPTH ? 1 : 0);
   constexpr int RS = rec_stride<Real, F>();
@@ -994,7 +996,7 @@ void fwd_launch(const Layout& L, const Real* bg, Real* out, unsigned char* ws,
     grid = dim3(min(n, L.B * L.NT * rg.S), 1);
     cudaMemsetAsync(&hdr->queue[0], 0, sizeof(uint32_t), st);
   }
-  kernel<<<grid, threads, smem, st>>>(
+  launch(kernel, grid, threads, smem, st,
       rg, table_of<Real>(ws, L.off_table), hdr,
       at<const uint2>(ws, L.off_ranges), at<const uint32_t>(ws, L.off_values),
       at<const Real>(ws, L.off_rec), bg, out, at<Real>(ws, L.off_tfinal),
@@ -1032,7 +1034,7 @@ void bwd_launch(const Layout& L, const Real* bg, const Real* dout, Real* dbg,
     grid = dim3(min(n, L.B * L.NT * rg.S), 1);
     cudaMemsetAsync(&hdr->queue[1], 0, sizeof(uint32_t), st);
   }
-  kernel<<<grid, threads, smem, st>>>(
+  launch(kernel, grid, threads, smem, st,
       rg, table_of<Real>(ws, L.off_table), hdr,
       at<const uint2>(ws, L.off_ranges), at<const uint32_t>(ws, L.off_values),
       at<const Real>(ws, L.off_rec), bg, dout, at<const Real>(ws, L.off_tfinal),

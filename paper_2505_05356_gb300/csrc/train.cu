@@ -32,6 +32,7 @@ __device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint64_t k) {
 __global__ void __launch_bounds__(256)
     train_begin_kernel(gftorf_train_state* st, float* bg, int n_bg, uint64_t seed,
                        uint64_t offset, uint64_t stride) {
+  grid_begin_early();
   __shared__ int64_t s_step;
   if (threadIdx.x == 0) {
     s_step = st->step + 1;
@@ -55,6 +56,7 @@ __global__ void __launch_bounds__(256)
     l2_loss_kernel(const float* __restrict__ out, const float* __restrict__ target,
                    float* __restrict__ grad, gftorf_train_state* st, int64_t n_rows,
                    int C, int FP, int64_t HW, float scale, double inv_m, int vec) {
+  grid_begin();
   float part = 0.f;
   if (vec) {
     const int64_t HW4 = HW >> 2;
@@ -109,6 +111,7 @@ struct AdamArgs {
 
 __global__ void __launch_bounds__(256)
     adam_kernel(AdamArgs a, const gftorf_train_state* __restrict__ st) {
+  grid_begin();
   const int64_t t = st->step > 0 ? st->step : 1;
   const float bc1 = 1.f - powf(a.b1, (float)t);
   const float bc2 = 1.f - powf(a.b2, (float)t);
@@ -147,7 +150,7 @@ extern "C" gftorf_status gftorf_train_begin_shard(gftorf_train_state* state, flo
     return GFTORF_ERR_ARG;
   if ((reinterpret_cast<uintptr_t>(state) & 7) != 0) return GFTORF_ERR_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  train_begin_kernel<<<1, 256, 0, st>>>(state, n_bg ? bg : nullptr, (int)n_bg, seed,
+  launch(train_begin_kernel, 1, 256, 0, st, state, n_bg ? bg : nullptr, (int)n_bg, seed,
                                         (uint64_t)bg_offset, (uint64_t)bg_stride);
   count_launches(1);
   return last_status();
@@ -175,7 +178,7 @@ extern "C" gftorf_status gftorf_l2_loss_scaled(const gftorf_dims* dims, const fl
                    (reinterpret_cast<uintptr_t>(target) & 15) == 0 &&
                    (reinterpret_cast<uintptr_t>(dL_dout) & 15) == 0;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  l2_loss_kernel<<<sm_count() * 8, 256, 0, st>>>(out, target, dL_dout, state, n_rows, L.C, FP,
+  launch(l2_loss_kernel, sm_count() * 8, 256, 0, st, out, target, dL_dout, state, n_rows, L.C, FP,
                                                  HW, (float)(2.0 / M), 1.0 / M, vec ? 1 : 0);
   count_launches(1);
   return last_status();
@@ -213,7 +216,7 @@ extern "C" gftorf_status gftorf_adam_step(const gftorf_adam_group* groups, int n
   const int64_t want = (most + 255) / 256;
   const int blocks = (int)(want < (int64_t)sm_count() * 8 ? want : (int64_t)sm_count() * 8);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  adam_kernel<<<blocks, 256, 0, st>>>(a, state);
+  launch(adam_kernel, blocks, 256, 0, st, a, state);
   count_launches(1);
   return last_status();
 }
