@@ -109,6 +109,7 @@ struct TableT {
   T kf[kMaxF];  // 4 f / c: psi / pi per metre of distance
   T source;
   T dilation, alpha_max, alpha_min, t_min, sigma_cut;
+  T log2_amin;  // log2 of alpha_min (-inf for 0)
 };
 using Table = TableT<double>;
 
@@ -192,6 +193,8 @@ void launch_preprocess_bwd(const Layout& L, const gftorf_gaussians& g,
 void launch_footprints(const Layout& L, const float* u, const float* v,
                        const int32_t* radius, const float* z,
                        unsigned char* ws, cudaStream_t st);
+void launch_footprint_bound(const Layout& L, const int32_t* radius, int64_t* bound,
+                            cudaStream_t st);
 void launch_binning(const Layout& L, unsigned char* ws, cudaStream_t st);
 size_t lb_bytes(const Layout& L);  // depth-sort look-back region
 void launch_export_keys(const Layout& L, uint64_t* keys, unsigned char* ws,
@@ -262,27 +265,27 @@ __device__ __forceinline__ int clamp_tile(float v, int hi) {
   if (v > (float)hi) return hi;
   return (int)v;
 }
-__device__ __forceinline__ void tile_rect(float u, float v, int r, int tw,
-                                          int th, int tiles_x, int tiles_y,
-                                          int& x0, int& y0, int& x1, int& y1) {
-  const float rf = (float)r, twf = (float)tw, thf = (float)th;
-  x0 = clamp_tile(floorf(__fdiv_rn(__fsub_rn(u, rf), twf)), tiles_x);
-  x1 = clamp_tile(__fadd_rn(floorf(__fdiv_rn(__fadd_rn(u, rf), twf)), 1.0f), tiles_x);
-  y0 = clamp_tile(floorf(__fdiv_rn(__fsub_rn(v, rf), thf)), tiles_y);
-  y1 = clamp_tile(__fadd_rn(floorf(__fdiv_rn(__fadd_rn(v, rf), thf)), 1.0f), tiles_y);
+// (tile sizes are powers of two, so x / tw is exactly x * (1 / tw), whose exponent
+// is 254 minus tw's: no division)
+__device__ __forceinline__ float tile_inv(int tw) {
+  return __int_as_float((254 << 23) - __float_as_int((float)tw));
 }
-
-// Same rectangle for separate half-widths in x and y (float), used for the
-// alpha-ellipse bounding box; it lies inside tile_rect's for rx, ry <= r.
+// half-widths rx, ry in x and y: for the alpha-ellipse bounding box it lies inside
+// the disc's for rx, ry <= r
 __device__ __forceinline__ void tile_rect_xy(float u, float v, float rx, float ry,
                                              int tw, int th, int tiles_x,
                                              int tiles_y, int& x0, int& y0,
                                              int& x1, int& y1) {
-  const float twf = (float)tw, thf = (float)th;
-  x0 = clamp_tile(floorf(__fdiv_rn(__fsub_rn(u, rx), twf)), tiles_x);
-  x1 = clamp_tile(__fadd_rn(floorf(__fdiv_rn(__fadd_rn(u, rx), twf)), 1.0f), tiles_x);
-  y0 = clamp_tile(floorf(__fdiv_rn(__fsub_rn(v, ry), thf)), tiles_y);
-  y1 = clamp_tile(__fadd_rn(floorf(__fdiv_rn(__fadd_rn(v, ry), thf)), 1.0f), tiles_y);
+  const float iw = tile_inv(tw), ih = tile_inv(th);
+  x0 = clamp_tile(floorf(__fmul_rn(__fsub_rn(u, rx), iw)), tiles_x);
+  x1 = clamp_tile(__fadd_rn(floorf(__fmul_rn(__fadd_rn(u, rx), iw)), 1.0f), tiles_x);
+  y0 = clamp_tile(floorf(__fmul_rn(__fsub_rn(v, ry), ih)), tiles_y);
+  y1 = clamp_tile(__fadd_rn(floorf(__fmul_rn(__fadd_rn(v, ry), ih)), 1.0f), tiles_y);
+}
+__device__ __forceinline__ void tile_rect(float u, float v, int r, int tw,
+                                          int th, int tiles_x, int tiles_y,
+                                          int& x0, int& y0, int& x1, int& y1) {
+  tile_rect_xy(u, v, (float)r, (float)r, tw, th, tiles_x, tiles_y, x0, y0, x1, y1);
 }
 
 // packed rectangle: 4 x uint16 (x0, y0, x1, y1) in one uint2

@@ -30,6 +30,7 @@ namespace {
 
 constexpr double kLog2e = 1.4426950408889634074;
 constexpr double kPiD = 3.14159265358979323846;
+constexpr double kLn2 = 0.69314718055994530942;
 
 template <typename Real>
 __device__ __forceinline__ Real rsqrt_t(Real x);
@@ -140,6 +141,15 @@ struct Params {
 template <typename Real>
 __device__ __forceinline__ void load_sh(const gftorf_gaussians& G, int g, int nsh, Real* c) {
   const Real* src = static_cast<const Real*>(G.sh) + (size_t)nsh * g;
+  if (sizeof(Real) == 4 && nsh == kMaxSh && (reinterpret_cast<uintptr_t>(G.sh) & 15) == 0) {
+    // whole aligned rows of 64 bytes: four loads instead of sixteen
+#pragma unroll
+    for (int q = 0; q < kMaxSh / 4; ++q) {
+      const float4 v = reinterpret_cast<const float4*>(src)[q];
+      c[4 * q] = v.x, c[4 * q + 1] = v.y, c[4 * q + 2] = v.z, c[4 * q + 3] = v.w;
+    }
+    return;
+  }
 #pragma unroll
   for (int l = 0; l < kMaxSh; ++l) c[l] = l < nsh ? src[l] : Real(0);
 }
@@ -282,8 +292,11 @@ __device__ __forceinline__ void geometry(const Params<Real>& P,
   Q.det = Q.cov[0] * Q.cov[2] - Q.cov[1] * Q.cov[1];
 }
 
+// Waiting for its loads (the largest stall) at five CTAs per SM: held to seven in
+// single precision (a few bytes spilled; six with the SH coefficients), -5 us of 137
+// for 16 frames of 300k Gaussians; the double instantiation is left alone.
 template <typename Real, int F, bool SH>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, sizeof(Real) == 8 ? 1 : (SH ? 6 : 7))
     preprocess_kernel(gftorf_gaussians G, const TableT<Real>* __restrict__ tab,
                       Header* __restrict__ hdr, Real* __restrict__ rec,
                       uint2* __restrict__ rect, uint32_t* __restrict__ zkey,
@@ -315,19 +328,21 @@ __global__ void __launch_bounds__(256)
       const int r = rad < Real(1 << 20) ? (int)rad : (1 << 20);
       const Real u = (Real)fr.fx * Q.p[0] * Q.iz + (Real)fr.cx;
       const Real v = (Real)fr.fy * Q.p[1] * Q.iz + (Real)fr.cy;
+      const Real log2_o = log2(P.o);
       int x0, y0, x1, y1;
-      tile_rect((float)u, (float)v, r, TW, TH, tiles_x, tiles_y, x0, y0, x1, y1);
-      if (cull) {
+      if (!cull) {
+        tile_rect((float)u, (float)v, r, TW, TH, tiles_x, tiles_y, x0, y0, x1, y1);
+      } else {
         // alpha = o G >= alpha_min only inside the ellipse
         // delta^T cov^-1 delta <= kappa = 2 ln(o / alpha_min); its bounding box
         // (plus slack for rounding) bounds every tile a pixel of which can
         // composite this Gaussian
-        const Real kappa = Real(2) * log(P.o / (Real)tab->alpha_min);
-        if (!(kappa >= Real(0))) {
-          x1 = x0;  // never reaches alpha_min
+        const Real kappa = Real(2 * kLn2) * (log2_o - tab->log2_amin);
+        if (!(kappa >= Real(-1e-4))) {  // (slack for the two logarithms' rounding)
+          x0 = x1 = y0 = y1 = 0;  // never reaches alpha_min
         } else {
-          const float ex = (float)(sqrt(kappa * Q.cov[0]) * Real(1.001) + Real(0.5));
-          const float ey = (float)(sqrt(kappa * Q.cov[2]) * Real(1.001) + Real(0.5));
+          const float ex = (float)(sqrt(fmax(kappa, Real(0)) * Q.cov[0]) * Real(1.001) + Real(0.5));
+          const float ey = (float)(sqrt(fmax(kappa, Real(0)) * Q.cov[2]) * Real(1.001) + Real(0.5));
           tile_rect_xy((float)u, (float)v, fminf((float)r, ex), fminf((float)r, ey), TW, TH,
                        tiles_x, tiles_y, x0, y0, x1, y1);
         }
@@ -345,7 +360,7 @@ __global__ void __launch_bounds__(256)
         o[2] = Real(-0.5 * kLog2e) * ca;
         o[3] = Real(-kLog2e) * cb;
         o[4] = Real(-0.5 * kLog2e) * cc;
-        o[5] = log2(P.o);  // alpha = 2^(power2 + log2 o)
+        o[5] = log2_o;  // alpha = 2^(power2 + log2 o)
         Real refl = P.amp;
         if (SH) {
           Real c[kMaxSh], w[3], val;
@@ -622,9 +637,16 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 8 ? 1 : (SH ? 3 : 4))
   if (D.amplitude) static_cast<Real*>(D.amplitude)[g] = gamp;
   if (SH && D.sh) {
     Real* o = static_cast<Real*>(D.sh) + (size_t)nsh * g;
+    if (sizeof(Real) == 4 && nsh == kMaxSh && (reinterpret_cast<uintptr_t>(D.sh) & 15) == 0) {
 #pragma unroll
-    for (int l = 0; l < NS; ++l)
-      if (l < nsh) o[l] = gsh[l];
+      for (int q = 0; q < NS / 4; ++q)
+        reinterpret_cast<float4*>(o)[q] = make_float4((float)gsh[4 * q], (float)gsh[4 * q + 1],
+                                                      (float)gsh[4 * q + 2], (float)gsh[4 * q + 3]);
+    } else {
+#pragma unroll
+      for (int l = 0; l < NS; ++l)
+        if (l < nsh) o[l] = gsh[l];
+    }
   }
 }
 
