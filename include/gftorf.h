@@ -281,6 +281,12 @@ gftorf_status gftorf_sort_footprints(const gftorf_dims* dims, const float* u,
                                      int64_t* count, void* workspace,
                                      size_t workspace_bytes, void* stream);
 
+/* An upper bound of the tile instances of such footprints (any centres), for
+ * sizing dims->max_instances: *bound (device int64) = the sum over [B][N] of
+ * (2r/tw + 2)(2r/th + 2), r = max(radius, 0).  Uses the same dims. */
+gftorf_status gftorf_footprint_bound(const gftorf_dims* dims, const int32_t* radius,
+                                     int64_t* bound, void* stream);
+
 /* gftorf_sort_footprints without a workspace argument, for callers that
  * cannot allocate device memory themselves: code running where cudaMalloc is
  * not available or not allowed (inside a region being captured into a CUDA

@@ -164,20 +164,38 @@ gftorf_status launch_status() {
   return e == cudaSuccess ? GFTORF_OK : GFTORF_ERR_CUDA;
 }
 
-// Writes the batch table into the workspace from a kernel argument, so the
-// upload is an ordinary kernel node inside a captured graph; clears the header too.
-__global__ void store_table_kernel(Table t, Table* dst, Header* hdr) {
+// The batch table as a kernel argument: NB frames and what follows them (a launch
+// copies its arguments several times, and all 64 frames are 25 KB).
+constexpr size_t kFrameWords = sizeof(FrameT<double>) / 8;
+constexpr size_t kTailWords = (sizeof(Table) - kMaxFrames * sizeof(FrameT<double>)) / 8;
+template <int NB>
+struct TableArg {
+  double w[NB * kFrameWords + kTailWords];
+};
+
+// Writes the batch table into the workspace from the argument, so the upload is an
+// ordinary kernel node inside a captured graph; clears the header too.
+template <int NB>
+__global__ void store_table_kernel(TableArg<NB> t, Table* dst, Header* hdr) {
   grid_begin_early();
   for (int i = threadIdx.x; i < (int)(sizeof(Header) / 4); i += blockDim.x)
     reinterpret_cast<uint32_t*>(hdr)[i] = 0u;
-  const int n = sizeof(Table) / sizeof(double);
-  const double* s = reinterpret_cast<const double*>(&t);
   double* d = reinterpret_cast<double*>(dst);
   float* f = reinterpret_cast<float*>(dst + 1);  // TableT<float>: same fields
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    d[i] = s[i];
-    f[i] = (float)s[i];
+  for (int i = threadIdx.x; i < (int)(NB * kFrameWords + kTailWords); i += blockDim.x) {
+    const int at = i < (int)(NB * kFrameWords) ? i : i + (int)((kMaxFrames - NB) * kFrameWords);
+    d[at] = t.w[i];
+    f[at] = (float)t.w[i];
   }
+}
+template <int NB>
+void store_table(const Table& t, const Layout& L, unsigned char* ws, cudaStream_t st) {
+  TableArg<NB> a;
+  const double* src = reinterpret_cast<const double*>(&t);
+  memcpy(a.w, src, NB * kFrameWords * 8);
+  memcpy(a.w + NB * kFrameWords, src + kMaxFrames * kFrameWords, kTailWords * 8);
+  launch(store_table_kernel<NB>, 1, 256, 0, st, a, at<Table>(ws, L.off_table),
+         at<Header>(ws, L.off_header));
 }
 
 bool finite(float x) { return isfinite(x) != 0; }
@@ -338,8 +356,12 @@ gftorf_status gftorf_preprocess(const gftorf_dims* dims,
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   unsigned char* ws = static_cast<unsigned char*>(workspace);
-  launch(store_table_kernel, 1, 256, 0, st, t, at<Table>(ws, L.off_table),
-         at<Header>(ws, L.off_header));
+  if (L.B <= 4)
+    store_table<4>(t, L, ws, st);
+  else if (L.B <= 16)
+    store_table<16>(t, L, ws, st);
+  else
+    store_table<kMaxFrames>(t, L, ws, st);
   count_launches(1);
   if (L.dtype == GFTORF_F32)
     launch_preprocess<float>(L, *g, ws, st);
@@ -462,6 +484,16 @@ gftorf_status gftorf_render_bwd(const gftorf_dims* dims,
   s = gftorf_composite_bwd(dims, bg, dL_dout, grads, workspace, workspace_bytes, stream);
   if (s != GFTORF_OK) return s;
   return gftorf_preprocess_bwd(dims, g, grads, workspace, workspace_bytes, stream);
+}
+
+gftorf_status gftorf_footprint_bound(const gftorf_dims* dims, const int32_t* radius,
+                                     int64_t* bound, void* stream) {
+  gftorf::TraceRange trace_("gftorf_footprint_bound");
+  if (!dims_ok(dims) || !bound || (dims->n_gaussians > 0 && !radius)) return GFTORF_ERR_ARG;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  cudaMemsetAsync(bound, 0, sizeof(int64_t), st);
+  launch_footprint_bound(make_layout(dims), radius, bound, st);
+  return launch_status();
 }
 
 gftorf_status gftorf_sort_footprints(const gftorf_dims* dims, const float* u,

@@ -145,6 +145,28 @@ __global__ void footprint_kernel(const float* __restrict__ u,
   if ((threadIdx.x & 31) == 0 && m) atomicAdd(&hdr->vis[b], (uint32_t)__popc(m));
 }
 
+// Most tiles that discs of the given radii can meet, summed
+__global__ void __launch_bounds__(256)
+    footprint_bound_kernel(const int32_t* __restrict__ radius, int64_t n, int TW, int TH,
+                           unsigned long long* __restrict__ bound) {
+  grid_begin_early();
+  __shared__ unsigned long long s_sum[8];
+  unsigned long long sum = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t d = 2u * (uint32_t)max(radius[i], 0);  // below 2^32
+    sum += (unsigned long long)(d / (uint32_t)TW + 2u) * (d / (uint32_t)TH + 2u);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) sum += s_sum[w];
+    if (sum) atomicAdd(bound, sum);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // depth sort: stable LSD radix sort, 8-bit digits, one segment per frame.
 // The per-frame digit totals of all four passes come from one reading of the
@@ -628,6 +650,16 @@ void launch_footprints(const Layout& L, const float* u, const float* v,
   launch(footprint_kernel, grid, 256, 0, st,
       u, v, radius, z, at<Header>(ws, L.off_header), at<uint2>(ws, L.off_rect),
       at<uint32_t>(ws, L.off_zkey), L.N, L.TW, L.TH, L.tiles_x, L.tiles_y);
+  count_launches(1);
+}
+
+void launch_footprint_bound(const Layout& L, const int32_t* radius, int64_t* bound,
+                            cudaStream_t st) {
+  const int64_t n = (int64_t)L.B * L.N;
+  if (n == 0) return;
+  const int blocks = (int)min((n + 1023) / 1024, (int64_t)(4 * sm_count()));
+  launch(footprint_bound_kernel, blocks, 256, 0, st, radius, n, L.TW, L.TH,
+         reinterpret_cast<unsigned long long*>(bound));
   count_launches(1);
 }
 

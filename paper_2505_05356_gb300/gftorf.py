@@ -115,6 +115,7 @@ def load(build_if_missing: bool = True):
     L.gftorf_render_fwd.argtypes = [_P(Dims), vp, vp, vp, sz, vp]
     L.gftorf_render_bwd.argtypes = [_P(Dims), _P(Gaussians), vp, vp, _P(Gradients), vp, sz, vp]
     L.gftorf_sort_footprints.argtypes = [_P(Dims), vp, vp, vp, vp, vp, vp, vp, vp, vp, sz, vp]
+    L.gftorf_footprint_bound.argtypes = [_P(Dims), vp, vp, vp]
     L.gftorf_export_tile_lists.argtypes = [_P(Dims), vp, vp, vp, vp, vp, sz, vp]
     L.gftorf_export_pixel_state.argtypes = [_P(Dims), vp, vp, vp, sz, vp]
     L.gftorf_read_device_status.argtypes = [_P(Dims), vp, sz, _P(ctypes.c_int64), vp]
@@ -140,7 +141,7 @@ def load(build_if_missing: bool = True):
     L.gftorf_adam_step.argtypes = [_P(AdamGroup), ctypes.c_int, ctypes.c_float, ctypes.c_float,
                                    ctypes.c_float, vp, vp]
     for name in ("gftorf_preprocess", "gftorf_render_fwd", "gftorf_render_bwd",
-                 "gftorf_sort_footprints", "gftorf_export_tile_lists",
+                 "gftorf_sort_footprints", "gftorf_footprint_bound", "gftorf_export_tile_lists",
                  "gftorf_export_pixel_state", "gftorf_read_device_status",
                  "gftorf_bin", "gftorf_composite_fwd", "gftorf_zero_grad_buffers",
                  "gftorf_composite_bwd", "gftorf_preprocess_bwd", "gftorf_train_begin",
@@ -169,11 +170,13 @@ def _ptr(t: Optional[torch.Tensor]):
         raise ValueError("expected a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError("expected a contiguous tensor")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()  # (ctypes takes an int where it wants a pointer)
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the current stream's handle without a Stream object around it (some 5 us per
+    # call, three calls per render)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _require_cuda():
@@ -459,8 +462,10 @@ def sort_footprints(u, v, radius, z, width, height, tile=(16, 16), max_instances
     L = load()
     B, n = u.shape
     if max_instances is None:
-        r = radius.to(torch.int64).clamp(min=0)
-        max_instances = int((((2 * r) // tile[0] + 2) * ((2 * r) // tile[1] + 2)).sum().item())
+        bound = torch.empty(1, dtype=torch.int64, device=u.device)
+        dims = Dims(n, B, width, height, tile[0], tile[1], 1, 1, F32, 0, 0, 0, 0)
+        code = L.gftorf_footprint_bound(ctypes.byref(dims), _ptr(radius), _ptr(bound), _stream())
+        max_instances = int(bound.item()) if code == OK else 1  # (the size below reports it)
     dims = Dims(n, B, width, height, tile[0], tile[1], 1, 1, F32, 0, 0, 0,
                 max_instances=max(1, max_instances))
     nbytes = L.gftorf_workspace_size(ctypes.byref(dims))
@@ -473,7 +478,7 @@ def sort_footprints(u, v, radius, z, width, height, tile=(16, 16), max_instances
     vals = torch.empty(cap, dtype=torch.int32, device=u.device)
     tiles = (-(-width // tile[0])) * (-(-height // tile[1]))
     ranges = torch.empty((B * tiles, 2), dtype=torch.int32, device=u.device)
-    count = torch.zeros(1, dtype=torch.int64, device=u.device)
+    count = torch.empty(1, dtype=torch.int64, device=u.device)
     _check(L.gftorf_sort_footprints(ctypes.byref(dims), _ptr(u), _ptr(v), _ptr(radius), _ptr(z),
                                     _ptr(keys), _ptr(vals), _ptr(ranges), _ptr(count),
                                     ctypes.c_void_p(ws.data_ptr() + off), nbytes, _stream()),
