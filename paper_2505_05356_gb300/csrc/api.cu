@@ -75,10 +75,13 @@ int default_ppt(const Layout& L) {
 }
 
 // Rows of the chunk counts' own region, and a region nothing uses: the sizes that an
-// earlier binning (chunks of instances, a scan of the Gaussians' tile counts) needed,
-// kept so that the fixed-scratch entry point takes and refuses the same problems.
+// earlier binning (chunks of instances, a scan of the Gaussians' tile counts, 512 bytes
+// more of header) needed, kept so that workspace sizes stay what they were and the
+// fixed-scratch entry point takes and refuses the same problems.
 size_t chunk_rows(const Layout& L) { return (size_t)((L.cap + 8191) / 8192) + L.B; }
-size_t spare_bytes(size_t BN) { return align_up(BN * 4 + 4) + ((BN + 16383) / 16384 + 1) * 8; }
+size_t spare_bytes(size_t BN) {
+  return 512 + align_up(BN * 4 + 4) + ((BN + 16383) / 16384 + 1) * 8;
+}
 
 // The chunk size and the counts' place: B n_chunk rows of NT words, in their own
 // region or, where that holds more, over the depth sort's ping-pong buffers and
