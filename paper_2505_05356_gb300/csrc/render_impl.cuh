@@ -152,8 +152,8 @@ __device__ __forceinline__ int butterfly_slot(int lane) {
 }
 
 // One CTA composites a CW x CH part of a binning tile (CW = min(TW, 32); CH =
-// 32 for tiles 32 or more wide, else TH): a 64x32 tile (whose list is shared)
-// is taken by S = 2 CTAs, a 64x64 one by 4, each testing the records against
+// 32, or 16 under narrow_parts(), for tiles 32 or more wide, else TH): a 64x32 tile (whose list is shared)
+// is taken by S = 2 (4) CTAs, a 64x64 one by 4 (8), each testing the records against
 // its own part, so each pixel composites the same records in the same order
 // as with 32x32 tiles.
 struct TileCtx {
@@ -393,24 +393,25 @@ __device__ __forceinline__ void log2_oG_column(const double* r, const Column<dou
 // Resident CTAs per SM the compiler is asked to fit (register budget).  Only
 // the 4-pixel variants are register limited: with 128 threads (16x32 tile) the
 // forward keeps 7 CTAs (<= 72 registers), the backward 6 (<= 80); with 256
-// threads (32x32 tile, WIDE) 3 of either (<= 85).
-template <int PPT, bool BWD, bool WIDE>
+// threads (32x32 part, WIDE = 1) 3 of either, with the 128 of a 32x16 part (WIDE =
+// 2) 6 (<= 85).
+template <int PPT, bool BWD, int WIDE>
 struct kMinBlocks {
   static constexpr int value =
-      WIDE ? 3 : (PPT == 4 ? (BWD ? 6 : 7) : (BWD ? (PPT == 2 ? 3 : 2) : 0));
+      WIDE ? 3 * WIDE : (PPT == 4 ? (BWD ? 6 : 7) : (BWD ? (PPT == 2 ? 3 : 2) : 0));
 };
-template <int PPT, bool WIDE>
+template <int PPT, int WIDE>
 struct kMaxThreads {
-  static constexpr int value = (WIDE ? 1024 : 512) / PPT;
+  static constexpr int value = (WIDE == 1 ? 1024 : 512) / PPT;
 };
-// threads of the CTA: a 32x32 part always has all of them, so that offsets in
+// threads of the CTA: a 32-wide part always has all of them, so that offsets in
 // its shared memory are constants instead of registers
-template <int PPT, bool WIDE>
+template <int PPT, int WIDE>
 __device__ __forceinline__ int cta_threads() {
   return WIDE ? kMaxThreads<PPT, WIDE>::value : (int)blockDim.x;
 }
 
-template <typename Real, int F, int PPT, bool DEPTH, bool COUNT, bool WIDE>
+template <typename Real, int F, int PPT, bool DEPTH, bool COUNT, int WIDE>
 __device__ __forceinline__ void render_tile_fwd(
     const TileCtx& tc, const RenderGeom& rg, const TableT<Real>* __restrict__ tab,
     const uint2* __restrict__ ranges, const uint32_t* __restrict__ values,
@@ -580,7 +581,7 @@ __device__ __forceinline__ void render_tile_fwd(
   }
 }
 
-template <typename Real, int F, int PPT, bool DEPTH, bool COUNT, bool WIDE>
+template <typename Real, int F, int PPT, bool DEPTH, bool COUNT, int WIDE>
 __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
                                   kMinBlocks<PPT, false, WIDE>::value)
     render_fwd_kernel(RenderGeom rg, const TableT<Real>* __restrict__ tab,
@@ -621,7 +622,7 @@ __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
 // ---------------------------------------------------------------------------
 // backward
 // ---------------------------------------------------------------------------
-template <typename Real, int F, int PPT, bool DEPTH, bool WIDE>
+template <typename Real, int F, int PPT, bool DEPTH, int WIDE>
 __device__ __forceinline__ void render_tile_bwd(
     const TileCtx& tc, const RenderGeom& rg, const TableT<Real>* __restrict__ tab,
     const uint2* __restrict__ ranges, const uint32_t* __restrict__ values,
@@ -909,7 +910,7 @@ __device__ __forceinline__ void render_tile_bwd(
   }
 }
 
-template <typename Real, int F, int PPT, bool DEPTH, bool WIDE>
+template <typename Real, int F, int PPT, bool DEPTH, int WIDE>
 __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
                                   kMinBlocks<PPT, true, WIDE>::value)
     render_bwd_kernel(RenderGeom rg, const TableT<Real>* __restrict__ tab,
@@ -957,13 +958,27 @@ __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
   }
 }
 
+// Whether tiles 32 or more wide are composited in 32x16 parts (128 threads, six per
+// SM) instead of 32x32 ones (256, three): the SMs fill more evenly and a CTA's
+// slowest warp holds three others up, not seven, but twice as many CTAs stage every
+// list entry.  16 frames of 640x480 (4800 parts of 32x32, over ten times what is
+// resident): 2030 -> 1990 us; one frame (300 parts): 235 -> 241 us, and
+// 8 frames at 640x576 with two frequencies (2880) no change, so from eight times on.
+// Every pixel composites the same records in the same order either way.  (Not in
+// double or when pairs are counted, whose kernels come with 256 threads alone.)
+bool narrow_parts(const Layout& L) {
+  if (L.TW < 32 || L.real_size != 4 || L.count_pairs) return false;
+  const int64_t parts = (int64_t)L.B * L.NT * (L.TW / 32) * (L.TH / 32);
+  return parts >= 8 * 152 * 3;
+}
+
 RenderGeom geom_of(const Layout& L) {
   RenderGeom g;
   g.N = L.N, g.W = L.W, g.H = L.H, g.TW = L.TW, g.TH = L.TH;
   g.tiles_x = L.tiles_x, g.NT = L.NT, g.P = L.P, g.C = L.C;
   g.rec_stride = L.rec_stride, g.B = L.B, g.cull = L.cull, g.phasor = L.phasor;
   g.CW = L.TW < 32 ? L.TW : 32;
-  g.CH = L.TW < 32 ? L.TH : 32;
+  g.CH = L.TW < 32 ? L.TH : (narrow_parts(L) ? 16 : 32);
   g.SX = L.TW / g.CW;
   g.S = g.SX * (L.TH / g.CH);
   return g;
@@ -976,7 +991,7 @@ int persistent_grid(KernelT kernel, int threads, size_t smem) {
   return sm_count() * (per_sm > 0 ? per_sm : 1);
 }
 
-template <typename Real, int F, int PPT, bool DEPTH, bool COUNT, bool WIDE>
+template <typename Real, int F, int PPT, bool DEPTH, bool COUNT, int WIDE>
 void fwd_launch(const Layout& L, const Real* bg, Real* out, unsigned char* ws,
                 cudaStream_t st) {
   constexpr int RS = rec_stride<Real, F>();
@@ -1008,7 +1023,7 @@ void fwd_launch(const Layout& L, const Real* bg, Real* out, unsigned char* ws,
 // four frequencies with the depth channel)
 constexpr int kMaxBwdSmem = 160 * 1024;
 
-template <typename Real, int F, int PPT, bool DEPTH, bool WIDE>
+template <typename Real, int F, int PPT, bool DEPTH, int WIDE>
 void bwd_launch(const Layout& L, const Real* bg, const Real* dout, Real* dbg,
                 unsigned char* ws, cudaStream_t st) {
   constexpr int NF = 2 * F + 1;
@@ -1046,26 +1061,32 @@ void bwd_launch(const Layout& L, const Real* bg, const Real* dout, Real* dbg,
 template <typename Real, int F, bool DEPTH>
 void fwd_dispatch(const Layout& L, const Real* bg, Real* out, unsigned char* ws,
                   cudaStream_t st) {
-  // 32-wide tiles come with 4 pixels per thread (256 threads)
+  // 32-wide tiles come with 4 pixels per thread (256 or 128 threads)
   if (L.TW > 16) {
-    if (L.count_pairs)
-      fwd_launch<Real, F, 4, DEPTH, true, true>(L, bg, out, ws, st);
-    else
-      fwd_launch<Real, F, 4, DEPTH, false, true>(L, bg, out, ws, st);
+    if (L.count_pairs) {
+      fwd_launch<Real, F, 4, DEPTH, true, 1>(L, bg, out, ws, st);
+      return;
+    }
+    if constexpr (sizeof(Real) == 4)
+      if (narrow_parts(L)) {
+        fwd_launch<Real, F, 4, DEPTH, false, 2>(L, bg, out, ws, st);
+        return;
+      }
+    fwd_launch<Real, F, 4, DEPTH, false, 1>(L, bg, out, ws, st);
     return;
   }
   if (L.count_pairs) {
     switch (L.ppt) {
-      case 1: fwd_launch<Real, F, 1, DEPTH, true, false>(L, bg, out, ws, st); break;
-      case 4: fwd_launch<Real, F, 4, DEPTH, true, false>(L, bg, out, ws, st); break;
-      default: fwd_launch<Real, F, 2, DEPTH, true, false>(L, bg, out, ws, st); break;
+      case 1: fwd_launch<Real, F, 1, DEPTH, true, 0>(L, bg, out, ws, st); break;
+      case 4: fwd_launch<Real, F, 4, DEPTH, true, 0>(L, bg, out, ws, st); break;
+      default: fwd_launch<Real, F, 2, DEPTH, true, 0>(L, bg, out, ws, st); break;
     }
     return;
   }
   switch (L.ppt) {
-    case 1: fwd_launch<Real, F, 1, DEPTH, false, false>(L, bg, out, ws, st); break;
-    case 4: fwd_launch<Real, F, 4, DEPTH, false, false>(L, bg, out, ws, st); break;
-    default: fwd_launch<Real, F, 2, DEPTH, false, false>(L, bg, out, ws, st); break;
+    case 1: fwd_launch<Real, F, 1, DEPTH, false, 0>(L, bg, out, ws, st); break;
+    case 4: fwd_launch<Real, F, 4, DEPTH, false, 0>(L, bg, out, ws, st); break;
+    default: fwd_launch<Real, F, 2, DEPTH, false, 0>(L, bg, out, ws, st); break;
   }
 }
 
@@ -1073,13 +1094,18 @@ template <typename Real, int F, bool DEPTH>
 void bwd_dispatch(const Layout& L, const Real* bg, const Real* dout, Real* dbg,
                   unsigned char* ws, cudaStream_t st) {
   if (L.TW > 16) {
-    bwd_launch<Real, F, 4, DEPTH, true>(L, bg, dout, dbg, ws, st);
+    if constexpr (sizeof(Real) == 4)
+      if (narrow_parts(L)) {
+        bwd_launch<Real, F, 4, DEPTH, 2>(L, bg, dout, dbg, ws, st);
+        return;
+      }
+    bwd_launch<Real, F, 4, DEPTH, 1>(L, bg, dout, dbg, ws, st);
     return;
   }
   switch (L.ppt) {
-    case 1: bwd_launch<Real, F, 1, DEPTH, false>(L, bg, dout, dbg, ws, st); break;
-    case 4: bwd_launch<Real, F, 4, DEPTH, false>(L, bg, dout, dbg, ws, st); break;
-    default: bwd_launch<Real, F, 2, DEPTH, false>(L, bg, dout, dbg, ws, st); break;
+    case 1: bwd_launch<Real, F, 1, DEPTH, 0>(L, bg, dout, dbg, ws, st); break;
+    case 4: bwd_launch<Real, F, 4, DEPTH, 0>(L, bg, dout, dbg, ws, st); break;
+    default: bwd_launch<Real, F, 2, DEPTH, 0>(L, bg, dout, dbg, ws, st); break;
   }
 }
 
