@@ -354,7 +354,6 @@ gftorf_status gftorf_preprocess(const gftorf_dims* dims,
     return GFTORF_ERR_ARG;
   t.dilation = consts->dilation, t.alpha_max = consts->alpha_max;
   t.alpha_min = consts->alpha_min, t.t_min = consts->t_min;
-  t.log2_amin = log2((double)consts->alpha_min);
   t.sigma_cut = consts->sigma_cut;
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);

@@ -109,7 +109,6 @@ struct TableT {
   T kf[kMaxF];  // 4 f / c: psi / pi per metre of distance
   T source;
   T dilation, alpha_max, alpha_min, t_min, sigma_cut;
-  T log2_amin;  // log2 of alpha_min (-inf for 0)
 };
 using Table = TableT<double>;
 

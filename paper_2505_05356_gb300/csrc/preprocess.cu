@@ -30,7 +30,6 @@ namespace {
 
 constexpr double kLog2e = 1.4426950408889634074;
 constexpr double kPiD = 3.14159265358979323846;
-constexpr double kLn2 = 0.69314718055994530942;
 
 template <typename Real>
 __device__ __forceinline__ Real rsqrt_t(Real x);
@@ -328,7 +327,6 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 8 ? 1 : (SH ? 6 : 7))
       const int r = rad < Real(1 << 20) ? (int)rad : (1 << 20);
       const Real u = (Real)fr.fx * Q.p[0] * Q.iz + (Real)fr.cx;
       const Real v = (Real)fr.fy * Q.p[1] * Q.iz + (Real)fr.cy;
-      const Real log2_o = log2(P.o);
       int x0, y0, x1, y1;
       if (!cull) {
         tile_rect((float)u, (float)v, r, TW, TH, tiles_x, tiles_y, x0, y0, x1, y1);
@@ -337,12 +335,14 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 8 ? 1 : (SH ? 6 : 7))
         // delta^T cov^-1 delta <= kappa = 2 ln(o / alpha_min); its bounding box
         // (plus slack for rounding) bounds every tile a pixel of which can
         // composite this Gaussian
-        const Real kappa = Real(2 * kLn2) * (log2_o - tab->log2_amin);
-        if (!(kappa >= Real(-1e-4))) {  // (slack for the two logarithms' rounding)
+        // (of the quotient, not a difference of logarithms: exactly the Gaussians
+        // with o < alpha_min have kappa < 0, whatever the rounding)
+        const Real kappa = Real(2) * log(P.o / (Real)tab->alpha_min);
+        if (!(kappa >= Real(0))) {
           x0 = x1 = y0 = y1 = 0;  // never reaches alpha_min
         } else {
-          const float ex = (float)(sqrt(fmax(kappa, Real(0)) * Q.cov[0]) * Real(1.001) + Real(0.5));
-          const float ey = (float)(sqrt(fmax(kappa, Real(0)) * Q.cov[2]) * Real(1.001) + Real(0.5));
+          const float ex = (float)(sqrt(kappa * Q.cov[0]) * Real(1.001) + Real(0.5));
+          const float ey = (float)(sqrt(kappa * Q.cov[2]) * Real(1.001) + Real(0.5));
           tile_rect_xy((float)u, (float)v, fminf((float)r, ex), fminf((float)r, ey), TW, TH,
                        tiles_x, tiles_y, x0, y0, x1, y1);
         }
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 8 ? 1 : (SH ? 6 : 7))
         o[2] = Real(-0.5 * kLog2e) * ca;
         o[3] = Real(-kLog2e) * cb;
         o[4] = Real(-0.5 * kLog2e) * cc;
-        o[5] = log2_o;  // alpha = 2^(power2 + log2 o)
+        o[5] = log2(P.o);  // alpha = 2^(power2 + log2 o)
         Real refl = P.amp;
         if (SH) {
           Real c[kMaxSh], w[3], val;
