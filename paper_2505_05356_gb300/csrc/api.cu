@@ -66,9 +66,13 @@ bool params_ok(const Layout& L, const gftorf_gaussians* g) {
 // resident warps on 152 SMs, one pixel per thread as long as all warps are resident
 // at once (3 frames of 96x64 pixels, fwd+bwd: 217 us with 2, 181 with 1), four where
 // they fill the GPU several times over (12 frames of 517x389, forward: 639 us with
-// 2, 622 with 4), else two.  Tiles 32 wide or more have four.
+// 2, 622 with 4), else two.  Tiles 32 wide or more have four.  In double always two:
+// its 512 threads of a 16x32 tile's one pixel each would need up to 210 KB of shared
+// memory, and its time is the FP64 units', not the warps' (one frame of 320x240: 806
+// us forward with 2, 889 with 1; 12 of 517x389: 15.4 ms with 2, 16.8 with 4).
 int default_ppt(const Layout& L) {
   if (L.TW >= 32) return 4;
+  if (L.dtype == GFTORF_F64) return 2;
   const int64_t resident = 152 * 24, warps1 = (int64_t)L.B * L.NT * (L.TW * L.TH / 32);
   if (warps1 <= resident) return 1;
   return warps1 >= 16 * resident && L.TW * L.TH / 4 >= 32 ? 4 : 2;

@@ -1019,8 +1019,8 @@ void fwd_launch(const Layout& L, const Real* bg, Real* out, unsigned char* ws,
   count_launches(1);
 }
 
-// dynamic shared memory of a backward CTA, at most (512 threads and 16 values:
-// four frequencies with the depth channel)
+// dynamic shared memory of a backward CTA, at most (single precision: 512 threads and
+// 16 values, four frequencies with the depth channel; double: 256 threads)
 constexpr int kMaxBwdSmem = 160 * 1024;
 
 template <typename Real, int F, int PPT, bool DEPTH, int WIDE>
