@@ -390,15 +390,24 @@ __device__ __forceinline__ void log2_oG_column(const double* r, const Column<dou
   }
 }
 
-// Resident CTAs per SM the compiler is asked to fit (register budget).  Only
-// the 4-pixel variants are register limited: with 128 threads (16x32 tile) the
-// forward keeps 7 CTAs (<= 72 registers), the backward 6 (<= 80); with 256
-// threads (32x32 part, WIDE = 1) 3 of either, with the 128 of a 32x16 part (WIDE =
-// 2) 6 (<= 85).
-template <int PPT, bool BWD, int WIDE>
+// Resident CTAs per SM the compiler is asked to fit (register budget).  With 4 pixels
+// per thread and 128 threads (16x32 tile) the forward keeps 7 CTAs (<= 72 registers),
+// the backward 6 (<= 80); with 256 threads (32x32 part, WIDE = 1) 3 of either, with the
+// 128 of a 32x16 part (WIDE = 2) 6 (<= 85).  The backward of four frequencies (15 or
+// 16 sums per record) spills 340-670 bytes at that and takes a third fewer warps with
+// 128 registers and no spills: 8 frames of 640x480, 32x32 tiles, 1323 -> 905 us, with
+// the depth channel 1448 -> 916; with three frequencies fewer warps were no gain on
+// 32x32 tiles (918 -> 950).  The single-precision backward of 2 pixels keeps 3 CTAs of
+// 256 threads (<= 85; uncapped, 8 frames at 16x16 with three frequencies: 867 -> 1013
+// us), that of 1 pixel 2 of 512 (<= 64; uncapped 1283 -> 1751).  In double a cap only
+// spills (one frame of 640x480, 2 pixels: 3729 us capped, 3364 not).
+template <typename Real, int F, int PPT, bool BWD, int WIDE>
 struct kMinBlocks {
+  static constexpr bool kFewer = BWD && sizeof(Real) == 4 && F == 4;
+  static constexpr int four = WIDE == 1 ? (kFewer ? 2 : 3)
+                                        : (kFewer ? 4 : (BWD || WIDE ? 6 : 7));
   static constexpr int value =
-      WIDE ? 3 * WIDE : (PPT == 4 ? (BWD ? 6 : 7) : (BWD ? (PPT == 2 ? 3 : 2) : 0));
+      PPT == 4 ? four : (!BWD || sizeof(Real) == 8 ? 0 : (PPT == 2 ? 3 : 2));
 };
 template <int PPT, int WIDE>
 struct kMaxThreads {
@@ -583,7 +592,7 @@ __device__ __forceinline__ void render_tile_fwd(
 
 template <typename Real, int F, int PPT, bool DEPTH, bool COUNT, int WIDE>
 __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
-                                  kMinBlocks<PPT, false, WIDE>::value)
+                                  kMinBlocks<Real, F, PPT, false, WIDE>::value)
     render_fwd_kernel(RenderGeom rg, const TableT<Real>* __restrict__ tab,
                       Header* __restrict__ hdr,
                       const uint2* __restrict__ ranges,
@@ -912,7 +921,7 @@ __device__ __forceinline__ void render_tile_bwd(
 
 template <typename Real, int F, int PPT, bool DEPTH, int WIDE>
 __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
-                                  kMinBlocks<PPT, true, WIDE>::value)
+                                  kMinBlocks<Real, F, PPT, true, WIDE>::value)
     render_bwd_kernel(RenderGeom rg, const TableT<Real>* __restrict__ tab,
                       Header* __restrict__ hdr,
                       const uint2* __restrict__ ranges,
