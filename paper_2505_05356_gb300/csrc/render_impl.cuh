@@ -129,8 +129,8 @@ struct Fold<LEN, 0> {
 template <int GS>
 constexpr int kRowRecords = 32 / GS;  // records whose values fit 32 rows
 template <typename Real, int GS>
-constexpr int row_floats() {  // per warp; the double instantiation folds by shuffles
-  return sizeof(Real) == 4 ? kRowRecords<GS> * GS * 32 : 0;
+constexpr int row_floats(int records) {  // per warp; the double instantiation folds by shuffles
+  return sizeof(Real) == 4 ? records * GS * 32 : 0;
 }
 
 // value index whose warp total lane `lane` ends with after Fold<GS, 16>;
@@ -639,7 +639,7 @@ __device__ __forceinline__ void render_tile_bwd(
     const Real* __restrict__ dout, const Real* __restrict__ tfinal,
     const uint32_t* __restrict__ nlast, Real* __restrict__ g2d, int g2d_stride,
     Real* __restrict__ dbg, Real* s_rec, Real* s_grad, uint32_t* s_id,
-    Real* s_red, int* s_cnt, Real* s_stage, unsigned* s_mask) {
+    Real* s_red, int* s_cnt, Real* s_stage, unsigned* s_mask, int row_records) {
   constexpr int NF = 2 * F + 1;
   constexpr int GS = 6 + NF + (DEPTH ? 1 : 0);
   constexpr int RS = rec_stride<Real, F>();
@@ -747,7 +747,9 @@ __device__ __forceinline__ void render_tile_bwd(
   // i % GS of the rows' record i / GS.  Double: shuffle butterfly.
   constexpr bool ROWS = sizeof(Real) == 4;
   const int red_slot = ROWS ? 0 : butterfly_slot<GS>(lane);
-  Real* const rows = s_stage + wid * row_floats<Real, GS>() + lane;  // this lane's column
+  // (how many records the rows hold: fewer than fit only with one pixel per thread)
+  const int records = PPT == 1 ? row_records : kRowRecords<GS>;
+  Real* const rows = s_stage + wid * row_floats<Real, GS>(records) + lane;  // this lane's column
   const Real ln2 = Real(kLn2);
   Real* gbase = g2d + (size_t)tc.b * rg.N * g2d_stride;
 
@@ -885,7 +887,7 @@ __device__ __forceinline__ void render_tile_bwd(
           for (int q = 0; q < GS; ++q) row[q * 32] = c[q];
           if ((unsigned)(lane - filled) < (unsigned)GS) red_dst = j * GS + lane - filled;
           filled += GS;
-          if (filled == kRowRecords<GS> * GS) add_rows();
+          if (filled == records * GS) add_rows();
         } else {
           Fold<GS, 16>::run(c, lane);
           if (red_slot >= 0 && c[0] != Real(0)) atomicAdd(&s_grad[j * GS + red_slot], c[0]);
@@ -930,7 +932,7 @@ __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
                       const Real* __restrict__ dout,
                       const Real* __restrict__ tfinal,
                       const uint32_t* __restrict__ nlast, Real* __restrict__ g2d,
-                      int g2d_stride, Real* __restrict__ dbg, int persistent) {
+                      int g2d_stride, Real* __restrict__ dbg, int persistent, int row_records) {
   grid_begin();
   constexpr int NF = 2 * F + 1;
   constexpr int GS = 6 + NF + (DEPTH ? 1 : 0);
@@ -950,7 +952,7 @@ __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
     render_tile_bwd<Real, F, PPT, DEPTH, WIDE>(tile_of(item, rg), rg, tab, ranges,
                                   values, rec, bg, dout, tfinal, nlast, g2d,
                                   g2d_stride, dbg, s_rec, s_grad, s_id, s_red, s_cnt,
-                                  s_stage, s_mask);
+                                  s_stage, s_mask, row_records);
     return;
   }
   __shared__ uint32_t s_item;
@@ -963,7 +965,7 @@ __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
     render_tile_bwd<Real, F, PPT, DEPTH, WIDE>(tile_of(item, rg), rg, tab, ranges,
                                   values, rec, bg, dout, tfinal, nlast, g2d,
                                   g2d_stride, dbg, s_rec, s_grad, s_id, s_red, s_cnt,
-                                  s_stage, s_mask);
+                                  s_stage, s_mask, row_records);
   }
 }
 
@@ -1031,6 +1033,9 @@ void fwd_launch(const Layout& L, const Real* bg, Real* out, unsigned char* ws,
 // dynamic shared memory of a backward CTA, at most (single precision: 512 threads and
 // 16 values, four frequencies with the depth channel; double: 256 threads)
 constexpr int kMaxBwdSmem = 160 * 1024;
+// shared memory of an SM, and of a backward CTA besides the dynamic part (masks,
+// counters, what the system takes)
+constexpr size_t kSmSmem = 228 * 1024, kCtaSmem = 2560;
 
 template <typename Real, int F, int PPT, bool DEPTH, int WIDE>
 void bwd_launch(const Layout& L, const Real* bg, const Real* dout, Real* dbg,
@@ -1042,9 +1047,21 @@ void bwd_launch(const Layout& L, const Real* bg, const Real* dout, Real* dbg,
   const int threads = rg.CW * rg.CH / PPT;
   // the records, their sums, the block scratch, an index per record, and the
   // stage slots or (after the staging barrier) the warps' rows
-  const size_t stage = (size_t)threads * RS, rows = (size_t)(threads / 32) * row_floats<Real, GS>();
-  const size_t smem = ((size_t)threads * (RS + GS) + 32 + (stage > rows ? stage : rows)) * sizeof(Real) +
-                      (size_t)threads * sizeof(uint32_t);
+  auto bytes = [&](int records) {
+    const size_t stage = (size_t)threads * RS,
+                 rows = (size_t)(threads / 32) * row_floats<Real, GS>(records);
+    return ((size_t)threads * (RS + GS) + 32 + (stage > rows ? stage : rows)) * sizeof(Real) +
+           (size_t)threads * sizeof(uint32_t);
+  };
+  // Rows of one record where those of several leave room for one CTA per SM instead of
+  // two and there are CTAs for two (three frequencies, a 16x32 tile's 512 threads; 8
+  // frames of 640x480: 1717 -> 1407 us; with few CTAs, one frame of 96x64, 117 -> 138)
+  int records = kRowRecords<GS>;
+  auto per_sm = [](size_t b) { return kSmSmem / (b + kCtaSmem); };
+  if (PPT == 1 && records > 1 && per_sm(bytes(records)) < 2 && per_sm(bytes(1)) >= 2 &&
+      L.B * L.NT * rg.S > sm_count())
+    records = 1;
+  const size_t smem = bytes(records);
   auto kernel = render_bwd_kernel<Real, F, PPT, DEPTH, WIDE>;
   static PerDeviceOnce attr;
   attr.run([&] {
@@ -1063,7 +1080,7 @@ void bwd_launch(const Layout& L, const Real* bg, const Real* dout, Real* dbg,
       at<const uint2>(ws, L.off_ranges), at<const uint32_t>(ws, L.off_values),
       at<const Real>(ws, L.off_rec), bg, dout, at<const Real>(ws, L.off_tfinal),
       at<const uint32_t>(ws, L.off_nlast), at<Real>(ws, L.off_g2d),
-      L.g2d_stride, dbg, L.mode == 1);
+      L.g2d_stride, dbg, L.mode == 1, records);
   count_launches(1);
 }
 

@@ -43,3 +43,8 @@ def test_four_frequencies_cost_little_more_than_three(tile, ppt):
     t3, t4 = _backward_us(3, tile, ppt), _backward_us(4, tile, ppt)
     assert t4 <= 1.35 * t3, (t3, t4)
 
+
+def test_one_pixel_per_thread_on_tall_tiles():
+    # the same sums from CTAs of 512 threads instead of 256
+    t16, t32 = _backward_us(3, (16, 16), 1), _backward_us(3, (16, 32), 1)
+    assert t32 <= 1.2 * t16, (t16, t32)
