@@ -430,6 +430,7 @@ __device__ __forceinline__ void render_tile_fwd(
   constexpr int NF = 2 * F + 1;
   constexpr int RS = rec_stride<Real, F>();
   constexpr unsigned ALL = (1u << PPT) - 1u;
+  constexpr bool BY_SIGN = sizeof(Real) == 4;  // how stopped pixels are told, below
   const int nthr = cta_threads<PPT, WIDE>(), tid = threadIdx.x;
   const ThreadPix tp = thread_pixels<PPT>(tid, rg.CW);
   const int lx = tp.lx, ly0 = tp.ly0;
@@ -456,8 +457,10 @@ __device__ __forceinline__ void render_tile_fwd(
     // T is kept negative in pixels that take no more records (outside, or
     // stopped): T (1 - alpha) is then below t_min and they are skipped by that
     // comparison alone, without a test of a done bit per pixel and record
-    // (with the constant CTA size: 588 -> 491 us for 16 frames of 300k Gaussians)
-    T[k] = outside & (1u << k) ? Real(-1) : Real(1);
+    // (with the constant CTA size: 588 -> 491 us for 16 frames of 300k Gaussians).
+    // In double the bit is tested, which spares the FP64 units what a stopped
+    // pixel would compute (8 frames of 640x480: 14.97 ms with the sign, 14.51)
+    T[k] = BY_SIGN && (outside & (1u << k)) ? Real(-1) : Real(1);
     accD[k] = 0;
     last[k] = range.x;
 #pragma unroll
@@ -530,6 +533,7 @@ __device__ __forceinline__ void render_tile_fwd(
         const uint32_t jn = get_index(r[kIdxWord<F>]) + 1;  // list entries up to this one
 #pragma unroll
         for (int k = 0; k < PPT; ++k) {
+          if (!BY_SIGN && (done & (1u << k))) continue;
           if (COUNT && !(done & (1u << k))) {
             ++evals;
             wevals += (m >> bit) & 1u;
@@ -540,7 +544,7 @@ __device__ __forceinline__ void render_tile_fwd(
           const Real tn = T[k] - aT;  // T (1 - alpha)
           if (tn < tmin) {
             done |= 1u << k;
-            T[k] = -fabs(T[k]);
+            if (BY_SIGN) T[k] = -fabs(T[k]);
             continue;
           }
           const Real w = aT * T[k];
@@ -568,7 +572,7 @@ __device__ __forceinline__ void render_tile_fwd(
 #pragma unroll
   for (int k = 0; k < PPT; ++k) {
     if (outside & (1u << k)) continue;
-    T[k] = fabs(T[k]);
+    if (BY_SIGN) T[k] = fabs(T[k]);
     const size_t pix = (size_t)(py0 + k) * rg.W + px;
     Real* o = out + (size_t)tc.b * rg.C * HW + pix;
     for (int f = 0; f < F; ++f)
