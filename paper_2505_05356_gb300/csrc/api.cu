@@ -96,11 +96,31 @@ void place_chunks(Layout& L) {
   const size_t dead = (L.off_ids2 - L.off_zkey2) / ((size_t)L.NT * 4), own = chunk_rows(L);
   const size_t rows = dead > own ? dead : own;
   if (dead > own) L.off_tcnt = L.off_zkey2;
-  L.chunk = 32;
-  L.chunks_per_cta = L.NT >= 512 ? 1 : (L.NT >= 64 ? 512 / L.NT : 8);
   auto per_frame = [&] { return ((size_t)L.N + L.chunk - 1) / L.chunk; };
-  while (L.chunk < kMaxChunk &&
-         per_frame() * L.B > (size_t)kMinChunkCtas * L.chunks_per_cta) L.chunk *= 2;
+  L.chunks_per_cta = L.NT >= kBlockTiles ? 1 : (L.NT >= 64 ? 512 / L.NT : 8);
+  if (L.NT >= kBlockTiles) {
+    // the fewest blocks whose columns and rows together are one word of 32 bits, or two
+    // where that would be kWideBlocks or more
+    for (int bits = 32; bits <= 64; bits += 32) {
+      if (L.n_block > 0 && L.n_block < kWideBlocks) break;
+      L.n_block = 0;
+      for (int nx = 1; nx <= L.tiles_x; ++nx) {
+        const int bw = (L.tiles_x + nx - 1) / nx;
+        if (bw >= bits) continue;
+        const int rows = bits - bw, ny = (L.tiles_y + rows - 1) / rows;
+        if (L.n_block > 0 && nx * ny >= L.n_block) continue;
+        L.bw = bw, L.bh = (L.tiles_y + ny - 1) / ny;
+        L.blocks_x = nx, L.n_block = nx * ny;
+      }
+    }
+  }
+  const size_t ctas = (size_t)kMinChunkCtas * L.chunks_per_cta;
+  const int most = L.n_block > 0 ? kMaxBlockChunk : kMaxChunk;
+  L.chunk = L.n_block > 0 ? 128 : 32;
+  while (L.chunk < most && per_frame() * L.B * (L.n_block > 0 ? L.n_block : 1) > ctas) L.chunk *= 2;
+  // (short lists, by the capacity: half as many rows are worth more than the CTAs)
+  if (L.n_block > 0 && L.chunk == most && (uint64_t)L.cap < 4 * per_frame() * L.B * L.NT)
+    L.chunk *= 2;
   while (per_frame() > 1 && per_frame() * L.B > rows) L.chunk *= 2;
   L.n_chunk = (int)(per_frame() > 0 ? per_frame() : 1);
 }

@@ -17,7 +17,7 @@
 //      tile column and row, the 32-bit mask of the group's Gaussians on it.  The
 //      Gaussians on a tile are the AND of its column's and its row's mask, in
 //      depth order from the lowest bit;
-//   3. per chunk (a run of groups of one frame, one warp), tile counts: the
+//   3. per chunk (a run of groups of one frame), tile counts: the
 //      masks' population counts summed over its groups; a scan over each frame's
 //      chunks per tile, and over all tiles, gives the tile ranges;
 //   4. scatter: the same masks again, each lane writing its tiles' Gaussians from
@@ -407,36 +407,47 @@ __global__ void __launch_bounds__(kSortThreads, 5)  // <= 48 registers, no spill
 // ---------------------------------------------------------------------------
 // chunk counts, column scan and scatter.  A chunk is L.chunk depth-consecutive
 // Gaussians of a frame (a multiple of 32); chunk c of frame b has row b n_chunk + c
-// of the counts.  A CTA takes L.chunks_per_cta chunks: its warps form the masks of
-// their groups, then every thread takes (chunk, tile) items, walking the chunk's
-// groups with the count or the cursor in a register.  Where the groups' masks
-// exceed the shared memory (very many tiles) they go in pieces, the items' values
-// waiting in the counts between two pieces.
+// of the counts.
+//
+// Small grids (below kBlockTiles tiles): a CTA takes L.chunks_per_cta chunks: its warps
+// form the masks of their groups over the whole grid, then every thread takes (chunk,
+// tile) items, walking the chunk's groups with the count or the cursor in a register.
 // (Chunks of instances, from a scan of the Gaussians' tile counts, with one
 // instance per lane and the lanes of one tile ranked by match.any, executed 4.4
 // instructions per instance on a chain of shared-memory cursor updates: scan,
 // count, column scan and scatter 144 us for 16 frames of 300k Gaussians at 64x64
-// tiles and 217 us for 12 frames of 120k at 16x16, now 109 and 159; one frame of
-// 100k at 32x32 51 and now 29.  One warp per chunk with its cursors in shared
-// memory instead of items: 116, 288, 46.)
+// tiles, now 109; one frame of 100k at 32x32 51 and now 29.  One warp per chunk with
+// its cursors in shared memory instead of items: 116, 46.)
+//
+// Larger grids: a CTA takes one chunk and one block of tiles, of at most 32 columns and
+// rows together (64 on grids of kWideBlocks such blocks and more), first packs those of
+// its Gaussians that meet the block, in order, and forms the masks of these alone, one
+// word (two) per lane and group of 32.  Over the whole grid the work grows with
+// Gaussians x tiles, whatever the footprints, and few CTAs do it where the space for
+// the counts allows few chunks: 300k Gaussians of radius 1 to 3 on 3840x2160 at 16x16
+// tiles, the whole binning 8255 us, in blocks 142; 12 frames of 120k on 517x389 at
+// 16x16 (lists of 40 tiles per Gaussian) 227 and 195; 16 of 300k at 32x32 (300 tiles)
+// 348 and 321.  At 180 tiles (64x32) a word holds nearly the grid.
 // ---------------------------------------------------------------------------
 struct ChunkArgs {
-  int N, NT, tiles_x, tiles_y, chunk, n_chunk, per_cta, piece;  // piece: groups at a time
+  int N, NT, tiles_x, tiles_y, chunk, n_chunk, per_cta;
+  int bw, bh, blocks_x, n_block;  // of the blocks of tiles (0: the whole grid)
 };
 
-// masks (and indices, if ids) of the CTA's groups [g0, g0 + n), group g the
-// Gaussians r0 + 32 g .. + 31 of the frame's depth order, empty from r1 on
-__device__ __forceinline__ void piece_masks(uint32_t* smem, int stride, const uint2* rc,
-                                            const uint32_t* id, int r0, int r1, int g0, int n,
-                                            int tiles_x, int words) {
+// masks (and indices, if ids) of the CTA's groups, group g the Gaussians r0 + 32 g ..
+// + 31 of the frame's depth order, empty from r1 on
+__device__ __forceinline__ void grid_masks(uint32_t* smem, int stride, const uint2* rc,
+                                           const uint32_t* id, int r0, int r1, int groups,
+                                           int tiles_x, int words) {
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int g = threadIdx.x >> 5; g < n; g += nw) {
-    const int r = r0 + 32 * (g0 + g) + lane;
+  for (int g = threadIdx.x >> 5; g < groups; g += nw) {
+    const int r = r0 + 32 * g + lane;
     uint32_t* m = smem + (size_t)g * stride;
     const uint2 rr = r < r1 ? rc[r] : make_uint2(0u, 0u);
     if (id) m[words + lane] = r < r1 ? id[r] : 0u;
     group_masks(m, rr, tiles_x, words, lane);
   }
+  __syncthreads();
 }
 
 constexpr int kBinThreads = 256;
@@ -451,46 +462,232 @@ __global__ void __launch_bounds__(kBinThreads)
   if (r0 >= r1) return;
   const int words = mask_words(a.tiles_x, a.tiles_y), per = a.chunk / 32;
   const int groups = (r1 - r0 + 31) / 32, chunks = (r1 - r0 + a.chunk - 1) / a.chunk;
-  const uint2* rc = srect + (size_t)b * a.N;
+  grid_masks(smem, words, srect + (size_t)b * a.N, nullptr, r0, r1, groups, a.tiles_x, words);
   uint32_t* rows = tcnt + ((size_t)b * a.n_chunk + c0) * a.NT;
-  for (int g0 = 0; g0 < groups; g0 += a.piece) {
-    const int n = min(a.piece, groups - g0);
-    __syncthreads();
-    piece_masks(smem, words, rc, nullptr, r0, r1, g0, n, a.tiles_x, words);
-    __syncthreads();
-    for (int i = threadIdx.x; i < chunks * a.NT; i += kBinThreads) {
-      const int c = i / a.NT, t = i - c * a.NT;
-      const int ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
-      const int lo = max(c * per - g0, 0), hi = min((c + 1) * per - g0, n);
-      if (lo >= hi) continue;
-      uint32_t acc = c * per < g0 ? rows[i] : 0u;
-      const uint32_t* m = smem + (size_t)lo * words;
-#pragma unroll 4
-      for (int g = lo; g < hi; ++g, m += words) acc += __popc(m[tx] & m[a.tiles_x + ty]);
-      rows[i] = acc;
+  for (int i = threadIdx.x; i < chunks * a.NT; i += kBinThreads) {
+    const int c = i / a.NT, t = i - c * a.NT;
+    const int ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
+    const int n = min(per, groups - c * per);
+    const uint32_t *col = smem + c * per * words + tx, *row = col - tx + a.tiles_x + ty;
+    uint32_t acc = 0;
+#pragma unroll 8
+    for (int g = 0; g < n; ++g, col += words, row += words) acc += __popc(*col & *row);
+    rows[i] = acc;
+  }
+}
+
+// A block of tiles [x, x + w) x [y, y + h)
+struct TileBlock {
+  int x, y, w, h;
+};
+__device__ __forceinline__ TileBlock tile_block(int k, const ChunkArgs& a) {
+  TileBlock t;
+  const int by = k / a.blocks_x;
+  t.x = (k - by * a.blocks_x) * a.bw;
+  t.y = by * a.bh;
+  t.w = min(a.bw, a.tiles_x - t.x);
+  t.h = min(a.bh, a.tiles_y - t.y);
+  return t;
+}
+// The tiles a thread takes of a block with W words of columns and rows (at most
+// 256 W^2 tiles): every 256th, as (column, row) in the block, and its index in the grid
+template <int W>
+struct OwnTiles {
+  int tx[W * W], ty[W * W], tile[W * W];
+  int n;
+  __device__ __forceinline__ OwnTiles(const TileBlock& t, int tiles_x) {
+    n = 0;
+#pragma unroll
+    for (int k = 0; k < W * W; ++k) {
+      const int i = (int)threadIdx.x + k * kBinThreads;
+      ty[k] = i / t.w;
+      tx[k] = i - ty[k] * t.w;
+      tile[k] = (t.y + ty[k]) * tiles_x + t.x + tx[k];
+      n += ty[k] < t.h ? 1 : 0;
     }
+  }
+};
+
+// The masks of those of the Gaussians [base, min(base + kBlockBatch, r1)) that meet the
+// block, packed in order: word S g + l is column l of group g, or row l - w (W words of
+// 32), and word S g + 64 + l the index of its l-th Gaussian (S = 96 words, with indices,
+// or 64).
+// Returns the number of groups; the whole CTA calls it, and may read the words until it
+// calls again.  `in` holds the batch's rectangles and indices and gets the next one's,
+// loaded while this one is worked on.
+constexpr int kBlockBatch = 4 * kBinThreads;
+template <int S>
+struct BlockBatch {
+  uint2 rect[4];  // four groups of 32 consecutive Gaussians per warp
+  uint32_t id[4];
+  __device__ __forceinline__ void load(const uint2* __restrict__ rc,
+                                       const uint32_t* __restrict__ ids, int base, int r1) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = base + warp * 128 + 32 * i + lane;
+      rect[i] = r < r1 ? rc[r] : make_uint2(0u, 0u);
+      if (S == 96) id[i] = r < r1 ? ids[r] : 0u;
+    }
+  }
+};
+template <int W, int S>
+__device__ __forceinline__ int block_masks(uint32_t* s_group, int* s_cnt, BlockBatch<S>& in,
+                                           const uint2* __restrict__ rc,
+                                           const uint32_t* __restrict__ ids, int base, int r1,
+                                           const TileBlock& t) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // both coordinates of a corner at once, tiles being fewer than 2^15: the top bit of
+  // each half stays where first <= last tile of the block, or end > its first
+  constexpr uint32_t kTop = 0x80008000u;
+  const uint32_t last = (uint32_t)((t.x + t.w - 1) | (t.y + t.h - 1) << 16) | kTop;
+  const uint32_t next = (uint32_t)((t.x + 1) | (t.y + 1) << 16);
+  unsigned kept[4];
+  int n = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint2 rr = in.rect[i];
+    const bool meets = ((last - rr.x) & ((rr.y | kTop) - next) & kTop) == kTop;
+    kept[i] = __ballot_sync(0xffffffffu, meets);
+    n += __popc(kept[i]);
+  }
+  if (lane == 0) s_cnt[warp] = n;
+  __syncthreads();  // (the previous batch's words have been read, too)
+  int pos = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < kBinThreads / 32; ++w) {
+    const int c = s_cnt[w];
+    pos += w < warp ? c : 0;
+    total += c;
+  }
+  if (n > 0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (kept[i] >> lane & 1u) {
+        const int at = pos + __popc(kept[i] & ((1u << lane) - 1u));
+        uint32_t* d = s_group + (at >> 5) * S + (at & 31);
+        d[0] = in.rect[i].x;
+        d[32] = in.rect[i].y;
+        if (S == 96) d[64] = in.id[i];
+      }
+      pos += __popc(kept[i]);
+    }
+  }
+  in.load(rc, ids, base + kBlockBatch, r1);
+  __syncthreads();
+  const int groups = (total + 31) / 32;
+  for (int g = warp; g < groups; g += kBinThreads / 32) {
+    uint32_t* d = s_group + g * S + lane;
+    int x0, y0, x1, y1;
+    unpack_rect(32 * g + lane < total ? make_uint2(d[0], d[32]) : make_uint2(0u, 0u), x0, y0, x1,
+                y1);
+    x0 = max(x0 - t.x, 0), x1 = min(x1 - t.x, t.w);
+    y0 = t.w + max(y0 - t.y, 0), y1 = t.w + min(y1 - t.y, t.h);
+    if (32 * g + lane >= total) x1 = x0 = 0, y1 = y0 = 0;
+#pragma unroll
+    for (int k = 0; k < W; ++k)
+      d[32 * k] = transpose32(span_word(x0, x1, k) | span_word(y0, y1, k), lane);
+  }
+  __syncthreads();
+  return groups;
+}
+
+template <int W>
+__global__ void __launch_bounds__(kBinThreads)
+    block_count_kernel(const uint2* __restrict__ srect, const Header* __restrict__ hdr,
+                       uint32_t* __restrict__ tcnt, uint64_t* __restrict__ sums, int n_sums,
+                       ChunkArgs a) {
+  grid_begin_early();
+  if (blockIdx.x == 0 && blockIdx.y == 0)  // for the column scan
+    for (int i = threadIdx.x; i < n_sums; i += kBinThreads) sums[i] = 0u;
+  __shared__ uint32_t s_group[kBlockBatch * 2];
+  __shared__ int s_cnt[kBinThreads / 32];
+  const int b = blockIdx.y, c = blockIdx.x / a.n_block, vis = (int)hdr->vis[b];
+  const int r0 = c * a.chunk, r1 = min(r0 + a.chunk, vis);
+  if (r0 >= r1) return;
+  const TileBlock t = tile_block(blockIdx.x - c * a.n_block, a);
+  const OwnTiles<W> own(t, a.tiles_x);
+  const uint2* rc = srect + (size_t)b * a.N;
+  uint32_t acc[W * W];
+#pragma unroll
+  for (int k = 0; k < W * W; ++k) acc[k] = 0;
+  BlockBatch<64> in;
+  in.load(rc, nullptr, r0, r1);
+  for (int base = r0; base < r1; base += kBlockBatch) {
+    const int groups = block_masks<W, 64>(s_group, s_cnt, in, rc, nullptr, base, r1, t);
+#pragma unroll
+    for (int k = 0; k < W * W; ++k) {
+      if (k >= own.n) break;
+      const uint32_t *col = s_group + own.tx[k], *row = s_group + t.w + own.ty[k];
+#pragma unroll 4
+      for (int g = 0; g < groups; ++g) acc[k] += __popc(col[64 * g] & row[64 * g]);
+    }
+  }
+  uint32_t* rows = tcnt + ((size_t)b * a.n_chunk + c) * a.NT;
+#pragma unroll
+  for (int k = 0; k < W * W; ++k)
+    if (k < own.n) rows[own.tile[k]] = acc[k];
+}
+
+// Exclusive scan over the CTA of four consecutive totals per thread, added to base;
+// base becomes the total's end, the same in every thread.
+constexpr int kColWarps = 32, kColWarpsMany = 8;
+constexpr int kScanTotals = 4 * 32 * kColWarps;  // per step
+__device__ __forceinline__ uint64_t scan_totals(const uint32_t* __restrict__ ttot, int i, int n,
+                                                uint32_t* v, uint64_t* s_w, uint64_t& base) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) v[k] = i + k < n ? __ldcg(&ttot[i + k]) : 0u;
+  const uint64_t mine = (uint64_t)v[0] + v[1] + v[2] + v[3];
+  uint64_t incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  __syncthreads();  // s_w has been read
+  if (lane == 31) s_w[w] = incl;
+  __syncthreads();
+  uint64_t st = base + incl - mine;
+  for (int k = 0; k < kColWarps; ++k) {
+    const uint64_t x = s_w[k];
+    base += x;
+    st += k < w ? x : 0u;
+  }
+  return st;
+}
+// the ranges of four consecutive tiles from the first one's start
+__device__ __forceinline__ void put_ranges(uint2* __restrict__ ranges, int i, int n, uint64_t st,
+                                           const uint32_t* v) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (i + k < n) ranges[i + k] = make_uint2((uint32_t)st, (uint32_t)(st + v[k]));
+    st += v[k];
   }
 }
 
 // per (frame, tile): exclusive prefix over the frame's chunks, and the tile's total.
 // A CTA covers 32 tiles (lanes, coalesced rows) and splits the frame's chunks into
-// kColWarps consecutive segments (warps): segment sums, then per-segment rescan.
-// The CTA that finishes last scans the totals of all (frame, tile) in order, which
-// gives the ranges and the instance count; lists that overflow the capacity are
-// left empty.
-constexpr int kColWarps = 32;
-__global__ void __launch_bounds__(32 * kColWarps)
+// WARPS consecutive segments (warps): segment sums, then per-segment rescan.
+// The CTA that finishes last makes the instance count, and with few tiles (kColWarps)
+// scans the totals of all (frame, tile) in order, which gives the ranges; lists that
+// overflow the capacity are left empty.  With many (kColWarpsMany) it scans only the sums of runs of
+// kScanTotals tiles, which the CTAs have added up, and tile_range_kernel makes the
+// ranges (16 frames of 8160 tiles, the binning: 514 -> 422 us; at five steps of
+// kScanTotals 207 -> 192).
+template <int WARPS>
+__global__ void __launch_bounds__(32 * WARPS)
     tile_colscan_kernel(uint32_t* __restrict__ tcnt, uint32_t* __restrict__ ttot,
-                        uint2* __restrict__ ranges, Header* __restrict__ hdr, ChunkArgs a,
-                        int64_t cap) {
+                        uint2* __restrict__ ranges, uint64_t* __restrict__ sums,
+                        Header* __restrict__ hdr, ChunkArgs a, int64_t cap) {
   grid_begin_early();
-  __shared__ uint32_t s_seg[kColWarps][32];
-  __shared__ uint64_t s_w[kColWarps];
+  __shared__ uint32_t s_seg[WARPS][32];
+  __shared__ uint64_t s_w[WARPS];
   __shared__ bool s_last;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int t = blockIdx.x * 32 + lane, b = blockIdx.y;
   const uint32_t n = ((uint32_t)hdr->vis[b] + a.chunk - 1) / a.chunk;
-  const uint32_t seg = (n + kColWarps - 1) / kColWarps;
+  const uint32_t seg = (n + WARPS - 1) / WARPS;
   const uint32_t s0 = min(n, (uint32_t)w * seg), s1 = min(n, (uint32_t)(w + 1) * seg);
   uint32_t* col = tcnt + (size_t)b * a.n_chunk * a.NT + t;
   uint32_t sum = 0;
@@ -509,48 +706,70 @@ __global__ void __launch_bounds__(32 * kColWarps)
       col[(size_t)c * a.NT] = run;
       run += v;
     }
-    if (w == kColWarps - 1) ttot[(size_t)b * a.NT + t] = run;
+    if (w == WARPS - 1) ttot[(size_t)b * a.NT + t] = run;
   }
-  if (w == kColWarps - 1) __threadfence();  // the totals' writers (the rest is for later kernels)
+  if (w == WARPS - 1) {
+    if constexpr (WARPS == kColWarpsMany) {  // (32 consecutive tiles lie in one run or in two)
+      const int i = b * a.NT + t, k = i / kScanTotals, k0 = __shfl_sync(0xffffffffu, k, 0);
+      uint64_t lo = t < a.NT && k == k0 ? run : 0u, hi = t < a.NT && k != k0 ? run : 0u;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        lo += __shfl_xor_sync(0xffffffffu, lo, o);
+        hi += __shfl_xor_sync(0xffffffffu, hi, o);
+      }
+      if (lane == 0) {
+        if (lo) atomicAdd(reinterpret_cast<unsigned long long*>(&sums[k0]), lo);
+        if (hi) atomicAdd(reinterpret_cast<unsigned long long*>(&sums[k0 + 1]), hi);
+      }
+    }
+    __threadfence();  // the totals' writers (the rest is for later kernels)
+  }
   __syncthreads();
   if (threadIdx.x == 0)
     s_last = atomicAdd(&hdr->col_done, 1u) == gridDim.x * gridDim.y - 1;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  // four consecutive totals per thread and step, scanned over the CTA
   const int total_tiles = gridDim.y * a.NT;
   uint64_t base = 0;
-  for (int i0 = 0; i0 < total_tiles; i0 += 4 * (int)blockDim.x) {
-    const int i = i0 + 4 * threadIdx.x;
-    uint32_t v[4];
+  if constexpr (WARPS == kColWarpsMany) {  // at most 800 runs: four per thread
+    const int runs = (total_tiles + kScanTotals - 1) / kScanTotals, i = 4 * (int)threadIdx.x;
+    uint64_t v[4], mine = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = i + k < total_tiles ? __ldcg(&ttot[i + k]) : 0u;
-    const uint64_t mine = (uint64_t)v[0] + v[1] + v[2] + v[3];
+    for (int k = 0; k < 4; ++k) {
+      v[k] = i + k < runs ? __ldcg(&sums[i + k]) : 0u;
+      mine += v[k];
+    }
     uint64_t incl = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint64_t y = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += y;
     }
-    __syncthreads();  // s_w has been read
     if (lane == 31) s_w[w] = incl;
     __syncthreads();
-    uint64_t st = base + incl - mine;
-    for (int k = 0; k < kColWarps; ++k) {
+    uint64_t st = incl - mine;
+    for (int k = 0; k < WARPS; ++k) {
       const uint64_t x = s_w[k];
       base += x;
       st += k < w ? x : 0u;
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      if (i + k < total_tiles) ranges[i + k] = make_uint2((uint32_t)st, (uint32_t)(st + v[k]));
+      if (i + k < runs) sums[i + k] = st;
       st += v[k];
+    }
+  } else {
+    for (int i0 = 0; i0 < total_tiles; i0 += kScanTotals) {
+      uint32_t v[4];
+      const int i = i0 + 4 * threadIdx.x;
+      const uint64_t st = scan_totals(ttot, i, total_tiles, v, s_w, base);
+      put_ranges(ranges, i, total_tiles, st, v);
     }
   }
   const bool over = base > (uint64_t)cap;  // (the same base in every thread)
-  if (over)
-    for (int i0 = 0; i0 < total_tiles; i0 += 4 * (int)blockDim.x)  // a thread's own ranges
+  if (over && WARPS == kColWarps)
+    for (int i0 = 0; i0 < total_tiles; i0 += kScanTotals)  // a thread's own ranges
       for (int k = 0; k < 4; ++k)
         if (i0 + 4 * (int)threadIdx.x + k < total_tiles)
           ranges[i0 + 4 * threadIdx.x + k] = make_uint2(0u, 0u);
@@ -561,9 +780,56 @@ __global__ void __launch_bounds__(32 * kColWarps)
   }
 }
 
+// the ranges of a run of kScanTotals tiles per CTA, from the run's start
+__global__ void __launch_bounds__(32 * kColWarps)
+    tile_range_kernel(const uint32_t* __restrict__ ttot, const uint64_t* __restrict__ sums,
+                      const Header* __restrict__ hdr, uint2* __restrict__ ranges, int total_tiles,
+                      int64_t cap) {
+  grid_begin_early();
+  __shared__ uint64_t s_w[kColWarps];
+  const int i = blockIdx.x * kScanTotals + 4 * threadIdx.x;
+  uint64_t base = sums[blockIdx.x];
+  uint32_t v[4];
+  uint64_t st = scan_totals(ttot, i, total_tiles, v, s_w, base);
+  if (hdr->count > cap) v[0] = v[1] = v[2] = v[3] = 0u, st = 0;
+  put_ranges(ranges, i, total_tiles, st, v);
+}
+
+// One tile's Gaussians of `groups` groups (column and row masks and indices `stride`
+// words apart) from values[p] on; returns the place after them.  Two Gaussians per
+// step and the next group's masks ahead: the loads of the indices and masks, not the
+// stores, are what the loop waits for (12 frames of 120k Gaussians at 16x16 tiles:
+// 129 -> 112 us).
+__device__ __forceinline__ uint32_t scatter_tile(const uint32_t* col, const uint32_t* row,
+                                                 const uint32_t* ids, int stride, int groups,
+                                                 uint32_t* __restrict__ values, uint32_t p,
+                                                 uint32_t cap) {
+  uint32_t next = groups > 0 ? *col & *row : 0u;
+  for (int g = 0; g < groups; ++g, ids += stride) {
+    uint32_t bits = next;
+    if (g + 1 < groups) {
+      col += stride;
+      row += stride;
+      next = *col & *row;
+    }
+    while (bits) {
+      const int k0 = __ffs(bits) - 1;
+      bits &= bits - 1;
+      const bool two = bits != 0;
+      const int k1 = two ? __ffs(bits) - 1 : k0;
+      bits &= bits - 1;  // (0 stays 0)
+      const uint32_t i0 = ids[k0], i1 = ids[k1];
+      if (p < cap) values[p] = i0;  // always, unless a sort wait timed out
+      if (two && p + 1 < cap) values[p + 1] = i1;
+      p += two ? 2 : 1;
+    }
+  }
+  return p;
+}
+
 __global__ void __launch_bounds__(kBinThreads)
     tile_scatter_kernel(const uint32_t* __restrict__ sorted_ids, const uint2* __restrict__ srect,
-                        const Header* __restrict__ hdr, uint32_t* __restrict__ tcnt,
+                        const Header* __restrict__ hdr, const uint32_t* __restrict__ tcnt,
                         const uint2* __restrict__ ranges, uint32_t* __restrict__ values,
                         ChunkArgs a, int64_t cap) {
   grid_begin();
@@ -573,49 +839,50 @@ __global__ void __launch_bounds__(kBinThreads)
   if (r0 >= r1 || hdr->count > cap) return;
   const int words = mask_words(a.tiles_x, a.tiles_y), per = a.chunk / 32, stride = words + 32;
   const int groups = (r1 - r0 + 31) / 32, chunks = (r1 - r0 + a.chunk - 1) / a.chunk;
-  const uint2* rc = srect + (size_t)b * a.N;
-  const uint32_t* id = sorted_ids + (size_t)b * a.N;
-  uint32_t* rows = tcnt + ((size_t)b * a.n_chunk + c0) * a.NT;
+  grid_masks(smem, stride, srect + (size_t)b * a.N, sorted_ids + (size_t)b * a.N, r0, r1, groups,
+             a.tiles_x, words);
+  const uint32_t* rows = tcnt + ((size_t)b * a.n_chunk + c0) * a.NT;
   const uint2* range = ranges + (size_t)b * a.NT;
-  const uint32_t capu = (uint32_t)cap;  // below 2^32
-  for (int g0 = 0; g0 < groups; g0 += a.piece) {
-    const int n = min(a.piece, groups - g0);
-    __syncthreads();
-    piece_masks(smem, stride, rc, id, r0, r1, g0, n, a.tiles_x, words);
-    __syncthreads();
-    for (int i = threadIdx.x; i < chunks * a.NT; i += kBinThreads) {
-      const int c = i / a.NT, t = i - c * a.NT;
-      const int ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
-      const int lo = max(c * per - g0, 0), hi = min((c + 1) * per - g0, n);
-      if (lo >= hi) continue;
-      uint32_t p = rows[i] + (c * per < g0 ? 0u : range[t].x);
-      // two Gaussians per step and the next group's masks ahead: the loads of the
-      // indices and masks, not the stores, are what the loop waits for (12 frames of
-      // 120k Gaussians at 16x16 tiles: 129 -> 112 us)
-      const uint32_t *col = smem + (size_t)lo * stride + tx,
-                     *row = smem + (size_t)lo * stride + a.tiles_x + ty,
-                     *ids = smem + (size_t)lo * stride + words;
-      uint32_t next = *col & *row;
-      for (int g = lo; g < hi; ++g, ids += stride) {
-        uint32_t bits = next;
-        if (g + 1 < hi) {
-          col += stride;
-          row += stride;
-          next = *col & *row;
-        }
-        while (bits) {
-          const int k0 = __ffs(bits) - 1;
-          bits &= bits - 1;
-          const bool two = bits != 0;
-          const int k1 = two ? __ffs(bits) - 1 : k0;
-          bits &= bits - 1;  // (0 stays 0)
-          const uint32_t i0 = ids[k0], i1 = ids[k1];
-          if (p < capu) values[p] = i0;  // always, unless a sort wait timed out
-          if (two && p + 1 < capu) values[p + 1] = i1;
-          p += two ? 2 : 1;
-        }
-      }
-      if (g0 + a.piece < groups) rows[i] = p;  // the next piece goes on from here
+  for (int i = threadIdx.x; i < chunks * a.NT; i += kBinThreads) {
+    const int c = i / a.NT, t = i - c * a.NT;
+    const int ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
+    const uint32_t* m = smem + (size_t)c * per * stride;
+    scatter_tile(m + tx, m + a.tiles_x + ty, m + words, stride, min(per, groups - c * per), values,
+                 rows[i] + range[t].x, (uint32_t)cap);
+  }
+}
+
+template <int W>
+__global__ void __launch_bounds__(kBinThreads)
+    block_scatter_kernel(const uint32_t* __restrict__ sorted_ids, const uint2* __restrict__ srect,
+                         const Header* __restrict__ hdr, const uint32_t* __restrict__ tcnt,
+                         const uint2* __restrict__ ranges, uint32_t* __restrict__ values,
+                         ChunkArgs a, int64_t cap) {
+  grid_begin();
+  __shared__ uint32_t s_group[kBlockBatch * 3];
+  __shared__ int s_cnt[kBinThreads / 32];
+  const int b = blockIdx.y, c = blockIdx.x / a.n_block, vis = (int)hdr->vis[b];
+  const int r0 = c * a.chunk, r1 = min(r0 + a.chunk, vis);
+  if (r0 >= r1 || hdr->count > cap) return;
+  const TileBlock t = tile_block(blockIdx.x - c * a.n_block, a);
+  const OwnTiles<W> own(t, a.tiles_x);
+  const uint32_t* rows = tcnt + ((size_t)b * a.n_chunk + c) * a.NT;
+  const uint2* range = ranges + (size_t)b * a.NT;
+  uint32_t p[W * W];
+#pragma unroll
+  for (int k = 0; k < W * W; ++k)
+    p[k] = k < own.n ? rows[own.tile[k]] + range[own.tile[k]].x : 0u;
+  const uint2* rc = srect + (size_t)b * a.N;
+  const uint32_t* ids = sorted_ids + (size_t)b * a.N;
+  BlockBatch<96> in;
+  in.load(rc, ids, r0, r1);
+  for (int base = r0; base < r1; base += kBlockBatch) {
+    const int groups = block_masks<W, 96>(s_group, s_cnt, in, rc, ids, base, r1, t);
+#pragma unroll
+    for (int k = 0; k < W * W; ++k) {
+      if (k >= own.n) break;
+      p[k] = scatter_tile(s_group + own.tx[k], s_group + t.w + own.ty[k], s_group + 64, 96, groups,
+                          values, p[k], (uint32_t)cap);
     }
   }
 }
@@ -637,7 +904,7 @@ __global__ void export_keys_kernel(const uint2* __restrict__ ranges,
 // look-back region: 64 words of per-pass tile counters, then one status word
 // per (pass, frame, tile, digit)
 constexpr size_t kLbCounters = 64;
-constexpr int kBinSmem = 40 * 1024;  // of a chunk kernel's masks at a time
+constexpr int kMaxScanSteps = 3;  // of the column scan's last CTA; beyond, tile_range_kernel
 size_t lb_bytes(const Layout& L) {
   return (kLbCounters + (size_t)4 * L.B * (L.n_dblk > 0 ? L.n_dblk : 1) * 256) * 4;
 }
@@ -701,22 +968,43 @@ void launch_binning(const Layout& L, unsigned char* ws, cudaStream_t st) {
     kin = kout[pass & 1];
     iin = iout[pass & 1];
   }
-  // 2.-3. per-chunk tile counts; per-frame column scan, totals and tile ranges
-  const int stride = mask_words(L.tiles_x, L.tiles_y) + 32;  // words per group, with indices
-  const int groups = L.chunks_per_cta * (L.chunk / 32);
-  const int piece = max(1, min(groups, kBinSmem / 4 / stride));
-  const ChunkArgs a{L.N, L.NT, L.tiles_x, L.tiles_y, L.chunk, L.n_chunk, L.chunks_per_cta, piece};
-  const dim3 ctas((L.n_chunk + L.chunks_per_cta - 1) / L.chunks_per_cta, L.B);
-  const size_t smem = (size_t)piece * stride * 4;
-  launch(tile_count_kernel, ctas, kBinThreads, smem, st, srect, hdr, tcnt, a);
-  launch(tile_colscan_kernel, dim3((L.NT + 31) / 32, L.B), 32 * kColWarps, 0, st,
-         tcnt, ttot, ranges,
-                                                                              hdr, a, L.cap);
+  // 2.-3. per-chunk tile counts; per-frame column scan, totals and tile ranges;
   // 4. stable scatter
-  launch(tile_scatter_kernel, ctas, kBinThreads, smem, st,
-         sorted, srect, hdr, tcnt, ranges, values, a,
-                                                       L.cap);
-  count_launches(9);
+  const ChunkArgs a{L.N,  L.NT, L.tiles_x, L.tiles_y,  L.chunk,  L.n_chunk, L.chunks_per_cta,
+                    L.bw, L.bh, L.blocks_x, L.n_block};
+  const dim3 col_ctas((L.NT + 31) / 32, L.B);
+  int launches = 9;
+  if (L.n_block > 0) {
+    const dim3 ctas(L.n_chunk * L.n_block, L.B);
+    const bool wide = L.bw + L.bh > 32;
+    const int tiles = L.B * L.NT, runs = (tiles + kScanTotals - 1) / kScanTotals;
+    // (over the sort's look-back words: 4 KB per frame and more, 8 bytes per 4096 tiles)
+    uint64_t* sums = runs > kMaxScanSteps ? reinterpret_cast<uint64_t*>(lb) : nullptr;
+    launch(wide ? block_count_kernel<2> : block_count_kernel<1>, ctas, kBinThreads, 0, st, srect,
+           hdr, tcnt, sums, sums ? runs : 0, a);
+    if (!sums) {
+      launch(tile_colscan_kernel<kColWarps>, col_ctas, 32 * kColWarps, 0, st, tcnt, ttot, ranges,
+             sums, hdr, a, L.cap);
+    } else {
+      launch(tile_colscan_kernel<kColWarpsMany>, col_ctas, 32 * kColWarpsMany, 0, st, tcnt, ttot,
+             ranges, sums, hdr, a, L.cap);
+      launch(tile_range_kernel, runs, 32 * kColWarps, 0, st, ttot, sums, hdr, ranges, tiles, L.cap);
+      ++launches;
+    }
+    launch(wide ? block_scatter_kernel<2> : block_scatter_kernel<1>, ctas, kBinThreads, 0, st,
+           sorted, srect, hdr, tcnt, ranges, values, a, L.cap);
+  } else {
+    // (at most 64 groups of at most 96 words and 32 indices: 32 KB)
+    const int stride = mask_words(L.tiles_x, L.tiles_y) + 32;  // words per group, with indices
+    const size_t smem = (size_t)L.chunks_per_cta * (L.chunk / 32) * stride * 4;
+    const dim3 ctas((L.n_chunk + L.chunks_per_cta - 1) / L.chunks_per_cta, L.B);
+    launch(tile_count_kernel, ctas, kBinThreads, smem, st, srect, hdr, tcnt, a);
+    launch(tile_colscan_kernel<kColWarps>, col_ctas, 32 * kColWarps, 0, st, tcnt, ttot, ranges,
+           nullptr, hdr, a, L.cap);
+    launch(tile_scatter_kernel, ctas, kBinThreads, smem, st, sorted, srect, hdr, tcnt, ranges,
+           values, a, L.cap);
+  }
+  count_launches(launches);
 }
 
 void launch_export_keys(const Layout& L, uint64_t* keys, unsigned char* ws,

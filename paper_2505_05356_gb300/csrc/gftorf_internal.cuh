@@ -79,10 +79,18 @@ constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;
-// Tile binning: at most kMaxChunk Gaussians per chunk where the counts' space allows,
-// and fewer, down to 32 (one group), where the batch would give the chunk kernels
-// less than about kMinChunkCtas CTAs (four per SM).
-constexpr int kMaxChunk = 256;
+// Tile binning: at most kMaxChunk Gaussians per chunk (kMaxBlockChunk where the grid is
+// taken in blocks, from kBlockTiles tiles on, twice that where the lists are short)
+// where the counts' space allows, and fewer, down to 32 (128), where the batch would
+// give the chunk kernels less than about kMinChunkCtas CTAs (four per SM of this part;
+// a constant, as the places in the workspace are the same without a device).  Chunks of
+// 2048 in blocks: 16 frames of 100k on 640x480 at 16x16, radius 1 to 3, 191 -> 176 us,
+// but radius 10 to 60, 387 -> 435.  Blocks of two words from kWideBlocks blocks of one
+// word on: at 32 the same Gaussians at 8x8 tiles (20 blocks) 254 -> 290 us, at 4 those
+// at 16x16 (6 blocks) 174 -> 189.
+constexpr int kMaxChunk = 256, kMaxBlockChunk = 1024;
+constexpr int kBlockTiles = 256;
+constexpr int kWideBlocks = 16;
 constexpr int kMinChunkCtas = 608;
 
 // Per-frame camera in device memory.
@@ -140,6 +148,7 @@ struct Layout {
   int chunk;       // Gaussians per binning chunk (a multiple of 32)
   int n_chunk;     // binning chunks per frame
   int chunks_per_cta;  // of the chunk kernels: enough for 512 (chunk, tile) items
+  int bw, bh, blocks_x, n_block;  // blocks of tiles (n_block 0: the whole grid at once)
   int64_t cap;
   size_t off_header, off_table, off_rec, off_rect, off_srect, off_zkey, off_zkey2,
       off_ids, off_ids2, off_dhist, off_dtot, off_spare, off_tcnt, off_ttot, off_ranges,
