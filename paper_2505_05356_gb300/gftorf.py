@@ -464,8 +464,9 @@ def sort_footprints(u, v, radius, z, width, height, tile=(16, 16), max_instances
     if max_instances is None:
         bound = torch.empty(1, dtype=torch.int64, device=u.device)
         dims = Dims(n, B, width, height, tile[0], tile[1], 1, 1, F32, 0, 0, 0, 0)
-        code = L.gftorf_footprint_bound(ctypes.byref(dims), _ptr(radius), _ptr(bound), _stream())
-        max_instances = int(bound.item()) if code == OK else 1  # (the size below reports it)
+        _check(L.gftorf_footprint_bound(ctypes.byref(dims), _ptr(radius), _ptr(bound), _stream()),
+               "gftorf_footprint_bound")
+        max_instances = int(bound.item())
     dims = Dims(n, B, width, height, tile[0], tile[1], 1, 1, F32, 0, 0, 0,
                 max_instances=max(1, max_instances))
     nbytes = L.gftorf_workspace_size(ctypes.byref(dims))
