@@ -99,19 +99,24 @@ typedef struct {
   int32_t n_frames;      /* B in [1, GFTORF_MAX_FRAMES]                     */
   int32_t width, height; /* image size in pixels, >= 1                      */
   int32_t tile_w, tile_h;/* one of 8x8, 16x16, 16x32, 32x32, 64x32, 64x64
-                            (w x h): the binning tile; a 64x32 or 64x64
-                            tile's list is composited by two or four CTAs
-                            of 32x32 pixels                               */
+                            (w x h): the binning tile; tiles 32 or more
+                            wide are composited in parts of 32x32 pixels,
+                            one CTA each, or of 32x16 in large
+                            single-precision batches                      */
   int32_t n_freq;        /* F in [1, GFTORF_MAX_FREQ]                       */
   int32_t n_offsets;     /* P in [1, GFTORF_MAX_OFFSETS]                    */
   int32_t dtype;         /* gftorf_dtype                                    */
   int32_t render_mode;   /* 0: one CTA per (frame, tile);
                             1: persistent CTAs over a (frame, tile) queue   */
-  int32_t pixels_per_thread; /* compositing pixels per thread: 1, 2 or 4
-                            (0: 2, or 4 for 32- and 64-wide tiles, which
-                            take only 4);
-                            tile_w * tile_h / it must be >= 32.  Results do
-                            not depend on it, nor on the tile shape.        */
+  int32_t pixels_per_thread; /* compositing pixels per thread: 1, 2 or 4;
+                            0: 4 for tiles 32 or more wide (which take only
+                            4), else 2 in double and 1, 2 or 4 by the
+                            batch's size in single precision.
+                            tile_w * tile_h / it must be >= 32 (for 0: / 2).
+                            Results do not depend on it, and on the tile
+                            shape only where alpha reaches alpha_min outside
+                            the sigma_cut square: a tile that it meets
+                            composites the Gaussian on all its pixels.      */
   int32_t flags;         /* GFTORF_FLAG_* bits, 0 for the defaults         */
   int32_t n_sh;          /* reflectivity model (Sec. 3): 0 = the scalar
                             gaussians.amplitude; 1, 4, 9 or 16 = real
@@ -350,7 +355,8 @@ int64_t gftorf_kernel_launches(void);
  * pixel, the entries of its tile's list up to and including the one that
  * stops it; counters[2] = the part of counters[1] in records that can reach
  * alpha_min in the rows of the pixel's warp (the compositing kernels skip the
- * others for the whole warp; the results do not depend on it).  Both are 0
+ * others for the whole warp; the results do not depend on it, this counter
+ * does on the pixels per thread, which shape a warp's block).  Both are 0
  * unless dims->flags has GFTORF_FLAG_COUNT_PAIRS.  counters: HOST int64[3]. */
 gftorf_status gftorf_read_counters(const gftorf_dims* dims, void* workspace,
                                    size_t workspace_bytes, int64_t* counters,

@@ -2,9 +2,11 @@
 
 Times one full step (preprocess, bin, composite, backward) of the caller's
 actual problem for every valid (tile shape, pixels per thread, grid or
-persistent compositing) and returns the fastest.  Results never change the
-rendered values (the forward is bit-identical across these choices, the
-gradients equal up to atomic summation order); only speed differs.
+persistent compositing) and returns the fastest.  For one tile shape the forward
+is bit-identical across these choices and the gradients equal up to atomic
+summation order; between tile shapes pixels differ where a Gaussian reaches
+alpha_min outside its sigma_cut square (a tile that the square meets composites
+it on all its pixels).
 """
 from __future__ import annotations
 
