@@ -62,18 +62,26 @@ bool params_ok(const Layout& L, const gftorf_gaussians* g) {
 }
 
 // Pixels per thread where the caller leaves the choice (the results do not depend on
-// it): 4 shares most of a record's work, 1 gives the most warps.  With about 24
-// resident warps on 152 SMs, one pixel per thread as long as all warps are resident
-// at once (3 frames of 96x64 pixels, fwd+bwd: 217 us with 2, 181 with 1), four where
-// they fill the GPU several times over (12 frames of 517x389, forward: 639 us with
-// 2, 622 with 4), else two.  Tiles 32 wide or more have four.  In double always two:
-// its 512 threads of a 16x32 tile's one pixel each would need up to 210 KB of shared
-// memory, and its time is the FP64 units', not the warps' (one frame of 320x240: 806
-// us forward with 2, 889 with 1; 12 of 517x389: 15.4 ms with 2, 16.8 with 4).
+// it): 4 shares most of a record's work, 1 gives the most warps.  Tiles 32 or more wide
+// have four.  In single precision, with about 24 resident warps per SM: one while all
+// warps of one pixel per thread are resident at once, four where they fill the GPU 16
+// times over, else two.  Forward + backward with 1 / 2 / 4 on 16x16 tiles, one frequency
+// (one to four frequencies and 16x32 tiles order alike, within 6 %):
+//   2400 warps (one frame of 320x240)     34+66   / 40+73   / 60+111 us
+//   4800                                  46+98   / 51+94   / 72+136
+//   7200                                  70+153  / 59+119  / 77+148
+//   19200 (two frames of 640x480)        116+243  / 92+196  / 102+204
+//   38400                                205+436  / 151+328 / 151+299
+//   67200                                340+735  / 243+542 / 233+484
+// (four wins from about 38400 on; with three frequencies from about 60000.)  In double
+// always two: its 512 threads of a 16x32 tile's one pixel each would need up to 210 KB
+// of shared memory, and its time is the FP64 units', not the warps' (one frame of
+// 320x240: 806 us forward with 2, 889 with 1; 12 of 517x389: 15.4 ms with 2, 16.8 with
+// 4).
 int default_ppt(const Layout& L) {
   if (L.TW >= 32) return 4;
   if (L.dtype == GFTORF_F64) return 2;
-  const int64_t resident = 152 * 24, warps1 = (int64_t)L.B * L.NT * (L.TW * L.TH / 32);
+  const int64_t resident = kSMs * 24, warps1 = (int64_t)L.B * L.NT * (L.TW * L.TH / 32);
   if (warps1 <= resident) return 1;
   return warps1 >= 16 * resident && L.TW * L.TH / 4 >= 32 ? 4 : 2;
 }

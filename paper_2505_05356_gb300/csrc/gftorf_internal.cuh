@@ -79,19 +79,23 @@ constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;
+// SMs of this part, where a rule over sizes needs them: a constant, not the device's
+// count, as layouts are made without a device and forward, backward and a captured
+// graph must take the same choice.
+constexpr int kSMs = 152;
+
 // Tile binning: at most kMaxChunk Gaussians per chunk (kMaxBlockChunk where the grid is
 // taken in blocks, from kBlockTiles tiles on, twice that where the lists are short)
 // where the counts' space allows, and fewer, down to 32 (128), where the batch would
-// give the chunk kernels less than about kMinChunkCtas CTAs (four per SM of this part;
-// a constant, as the places in the workspace are the same without a device).  Chunks of
-// 2048 in blocks: 16 frames of 100k on 640x480 at 16x16, radius 1 to 3, 191 -> 176 us,
-// but radius 10 to 60, 387 -> 435.  Blocks of two words from kWideBlocks blocks of one
-// word on: at 32 the same Gaussians at 8x8 tiles (20 blocks) 254 -> 290 us, at 4 those
-// at 16x16 (6 blocks) 174 -> 189.
+// give the chunk kernels less than about kMinChunkCtas CTAs.  Chunks of 2048 in
+// blocks: 16 frames of 100k on 640x480 at 16x16, radius 1 to 3, 191 -> 176 us, but
+// radius 10 to 60, 387 -> 435.  Blocks of two words from kWideBlocks blocks of one word
+// on: at 32 the same Gaussians at 8x8 tiles (20 blocks) 254 -> 290 us, at 4 those at
+// 16x16 (6 blocks) 174 -> 189.
 constexpr int kMaxChunk = 256, kMaxBlockChunk = 1024;
 constexpr int kBlockTiles = 256;
 constexpr int kWideBlocks = 16;
-constexpr int kMinChunkCtas = 608;
+constexpr int kMinChunkCtas = 4 * kSMs;
 
 // Per-frame camera in device memory.
 template <typename T>

@@ -457,15 +457,15 @@ __global__ void __launch_bounds__(192, MT == 2 ? 1 : 2)
               tma_load_2d(sa + j * 8192, &tmA, full0 + 8 * s, m0 * MT + 64 * j, (kb0 + i) * BK);
           } else {
             tma_load_2d(sa, &tmA, full0 + 8 * s, (kb0 + i) * BK, m0 * MT);
-        }
-        if (MNB) {
+          }
+          if (MNB) {
 #pragma unroll
-          for (int j = 0; j < BN / 64; ++j)
-            tma_load_2d(sa + A_BYTES + j * 8192, &tmB, full0 + 8 * s, n0 + 64 * j,
-                        (kb0 + i) * BK);
-        } else {
-          tma_load_2d(sa + A_BYTES, &tmB, full0 + 8 * s, (kb0 + i) * BK, n0);
-        }
+            for (int j = 0; j < BN / 64; ++j)
+              tma_load_2d(sa + A_BYTES + j * 8192, &tmB, full0 + 8 * s, n0 + 64 * j,
+                          (kb0 + i) * BK);
+          } else {
+            tma_load_2d(sa + A_BYTES, &tmB, full0 + 8 * s, (kb0 + i) * BK, n0);
+          }
         }
         __syncwarp();
         issued = i + 1;
@@ -970,9 +970,9 @@ __device__ __forceinline__ void epi_sync() {
 
 // What a training forward keeps for the backward (TRAIN): the encoded input
 // and every hidden activation (row-major BF16, stored by TMA from the tile in
-// shared memory through maps.enc / maps.act), and the ReLU masks as bits
-// ([layer][Mp][8] words) -- the same values the layer-by-layer forward
-// stores.  The stores of tile t are issued (and waited for before the tile is
+// shared memory through maps.enc / maps.act), and the ReLU masks as bits (per
+// layer Mp kW / 32 words, in the order of mask_at) -- the same values the
+// layer-by-layer forward stores.  The stores of tile t are issued (and waited for before the tile is
 // written again) by epilogue thread 32 t.
 struct FusedKeep {
   uint32_t* bits;
@@ -1078,7 +1078,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
           }
     }
   } else {
-    // epilogue warps: row r of every tile, a quarter of the columns
+    // epilogue warps: 32 rows of every tile (the encoding and the head: row r), half of
+    // the columns, as fragments
     const int q = warp & 3, part = warp >> 2;
     const int r = q * 32 + lane;
     uint32_t acc_ph[kPair] = {0, 0};
@@ -1200,7 +1201,7 @@ constexpr int kBwdSmem = kFusedSmem;
 
 struct FusedBwdArgs {
   const float* dd;      // dL/d(delta) [M][3]
-  const uint32_t* bits; // ReLU masks [layer][Mp][8]
+  const uint32_t* bits; // ReLU masks, per layer Mp kW / 32 words (mask_at)
   float* denc;          // [Mp][128] (out)
   int M, Mp, n_tiles;
 };
@@ -1599,7 +1600,7 @@ extern "C" gftorf_status gftorf_mlp_forward(int32_t n_gaussians, int32_t n_frame
   if (L.M == 0) return cudaGetLastError() == cudaSuccess ? GFTORF_OK : GFTORF_ERR_CUDA;
   auto* wb = ptr<__nv_bfloat16>(ws, L.off_wb);
   auto* wt = ptr<__nv_bfloat16>(ws, L.off_wt);
-  launch(mlp_prep_weights_kernel, 4 * 152, 256, 0, st, theta, wb, wt);
+  launch(mlp_prep_weights_kernel, 4 * kSMs, 256, 0, st, theta, wb, wt);
   Times tm;
   memset(&tm, 0, sizeof(tm));
   for (int b = 0; b < n_frames; ++b) tm.t[b] = times[b];
@@ -1624,13 +1625,13 @@ extern "C" gftorf_status gftorf_mlp_forward(int32_t n_gaussians, int32_t n_frame
     const int n_pairs = (mt + kPair - 1) / kPair;
     const int inj = g_inject.load();
     launch(mlp_fused_fwd_kernel<true>, n_pairs < sms ? n_pairs : sms, kFusedThreads, kFusedSmem, st,
-        maps, theta, means, tm, n_gaussians, L.M, mt, inv_scale, delta, status,
-        inj == 1 ? 50000000ull : 2000000000ull, inj == 1, keep);
+           maps, theta, means, tm, n_gaussians, L.M, mt, inv_scale, delta, status,
+           inj == 1 ? 50000000ull : 2000000000ull, inj == 1, keep);
     count_launches(2);
     return cudaGetLastError() == cudaSuccess ? GFTORF_OK : GFTORF_ERR_CUDA;
   }
   launch(mlp_encode_kernel, (Mp + 127) / 128, 128, 0, st, means, tm, n_gaussians, n_frames,
-                                                      inv_scale, Mp, enc);
+         inv_scale, Mp, enc);
   count_launches(2);
   for (int l = 0; l < kDepth; ++l) {
     const int K = l == 0 ? kIn : kW;
@@ -1691,7 +1692,7 @@ extern "C" gftorf_status gftorf_mlp_backward(int32_t n_gaussians, int32_t n_fram
   float* dwx = ptr<float>(ws, L.off_dwx);
   cudaMemsetAsync(dwx, 0, dwx_floats() * 4, st);
   if (L.M == 0) {
-    launch(mlp_unpack_grads_kernel, 4 * 152, 256, 0, st, dwx, d_theta);
+    launch(mlp_unpack_grads_kernel, 4 * kSMs, 256, 0, st, dwx, d_theta);
     count_launches(1);
     return cudaGetLastError() == cudaSuccess ? GFTORF_OK : GFTORF_ERR_CUDA;
   }
@@ -1718,9 +1719,8 @@ extern "C" gftorf_status gftorf_mlp_backward(int32_t n_gaussians, int32_t n_fram
   const unsigned long long wait_ns = inj_loads ? 50000000ull : 2000000000ull;
   const bool layerwise = g_inject.load(std::memory_order_relaxed) == 2;
   launch(mlp_head_grad_kernel, min((Mp + kHeadGradThreads - 1) / kHeadGradThreads, 4 * sms),
-         kHeadGradThreads, 0, st,
-         d_delta, L.M, Mp, layerwise ? dzh : nullptr,
-                                                    dzht, dbias_of(kDepth), kW + kExt);
+         kHeadGradThreads, 0, st, d_delta, L.M, Mp, layerwise ? dzh : nullptr, dzht,
+         dbias_of(kDepth), kW + kExt);
   count_launches(1);
   // head: dW_head += dZh^T H_7 (H_7 read MN-major)
   {
@@ -1803,14 +1803,13 @@ extern "C" gftorf_status gftorf_mlp_backward(int32_t n_gaussians, int32_t n_fram
     if (!(l == 0 ? gemm<kIn, EPI_PARTIAL, 2, 1, 1>(ma, mb, a, 1, 1, splits, st)
                  : gemm<kW, EPI_PARTIAL, 2, 1, 1>(ma, mb, a, 1, 1, splits, st)))
       return GFTORF_ERR_CUDA;
-    launch(mlp_reduce_dw_kernel, kW * K / 128, 32 * kReduceWarps, 0, st,
-           part, splits, K, dwx + dwx_off(l),
-                                                               K + kExt);
+    launch(mlp_reduce_dw_kernel, kW * K / 128, 32 * kReduceWarps, 0, st, part, splits, K,
+           dwx + dwx_off(l), K + kExt);
     count_launches(1);
   }
-  launch(mlp_unpack_grads_kernel, 4 * 152, 256, 0, st, dwx, d_theta);
+  launch(mlp_unpack_grads_kernel, 4 * kSMs, 256, 0, st, dwx, d_theta);
   launch(mlp_encode_bwd_kernel, (n_gaussians + 63) / 64, 128, 0, st, means, denc, n_gaussians,
-                                                               n_frames, inv_scale, d_means);
+         n_frames, inv_scale, d_means);
   count_launches(2);
   (void)times;
   return cudaGetLastError() == cudaSuccess ? GFTORF_OK : GFTORF_ERR_CUDA;
@@ -1877,7 +1876,7 @@ extern "C" gftorf_status gftorf_mlp_infer(int32_t n_gaussians, int32_t n_frames,
   if (M == 0) return cudaGetLastError() == cudaSuccess ? GFTORF_OK : GFTORF_ERR_CUDA;
   auto* wb = ptr<__nv_bfloat16>(workspace, 256);
   auto* wt = wb + wb_elems();
-  launch(mlp_prep_weights_kernel, 4 * 152, 256, 0, st, theta, wb, wt);
+  launch(mlp_prep_weights_kernel, 4 * kSMs, 256, 0, st, theta, wb, wt);
   FusedMaps maps;
   for (int l = 0; l <= kDepth; ++l) {
     const int K = l == 0 ? kIn : kW, rows = l == kDepth ? kHeadRows : kW;

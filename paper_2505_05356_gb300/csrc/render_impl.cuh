@@ -23,8 +23,8 @@
 //   alpha_k dL/dalpha_k = v - alpha_k / (1 - alpha_k) R,   R <- R + 2 v
 // with g_c the gradient of the accumulators (the raw samples are linear in
 // them) and g_T = sum_c bg_c dL/dQ_c.  Per-Gaussian sums over the CTA's
-// pixels: warp shuffle reduction, shared-memory accumulation, then one
-// global atomic per value per CTA.
+// pixels: per warp through rows of shared memory (in double by shuffles),
+// shared-memory accumulation, then one global atomic per value per CTA.
 #pragma once
 
 #include "gftorf_internal.cuh"
@@ -355,8 +355,6 @@ __device__ __forceinline__ float row_sum(const float* row, int lane) {
   unpack2(add2_rn(a, b), lo, hi);
   return lo + hi;
 }
-// (never called: the double instantiation folds by shuffles)
-__device__ __forceinline__ double row_sum(const double*, int) { return 0.0; }
 
 // log2_oG and dy of the PPT pixels of one column: pairs of pixels in packed FP32x2
 // (the same roundings as log2_oG); the double instantiation stays scalar
@@ -807,13 +805,15 @@ __device__ __forceinline__ void render_tile_bwd(
     __syncwarp();
     int filled = 0, red_dst = 0;  // rows in use; where this lane's sum goes
     auto add_rows = [&]() {
-      __syncwarp();
-      if (lane < filled) {
-        const Real t = row_sum(rows + lane * 31, lane);
-        if (t != Real(0)) atomicAdd(&s_grad[red_dst], t);
+      if constexpr (ROWS) {
+        __syncwarp();
+        if (lane < filled) {
+          const Real t = row_sum(rows + lane * 31, lane);
+          if (t != Real(0)) atomicAdd(&s_grad[red_dst], t);
+        }
+        __syncwarp();
+        filled = 0;
       }
-      __syncwarp();
-      filled = 0;
     };
     for (int q = nq - 1; q >= 0; --q) {
      unsigned m = s_mask[wid * kMaskWords + q];
@@ -976,15 +976,18 @@ __global__ void __launch_bounds__(kMaxThreads<PPT, WIDE>::value,
 // Whether tiles 32 or more wide are composited in 32x16 parts (128 threads, six per
 // SM) instead of 32x32 ones (256, three): the SMs fill more evenly and a CTA's
 // slowest warp holds three others up, not seven, but twice as many CTAs stage every
-// list entry.  16 frames of 640x480 (4800 parts of 32x32, over ten times what is
-// resident): 2030 -> 1990 us; one frame (300 parts): 235 -> 241 us, and
-// 8 frames at 640x576 with two frequencies (2880) no change, so from eight times on.
-// Every pixel composites the same records in the same order either way.  (Not in
-// double or when pairs are counted, whose kernels come with 256 threads alone.)
+// list entry.  Forward + backward, 640x480 at 32x32 tiles, one / two / four frequencies:
+// 16 frames (4800 parts) 1495 us against 1499, 1881 / 1882, 2480 / 2519; 12 frames
+// (3600) 1151 / 1158, 1445 / 1463, 1902 / 1943; 8 (2400) 806 / 818, 1027 / 1035, 1336 /
+// 1363; 4 (1200) 460 / 454, 563 / 569, 736 / 739; one frame (300) 241 / 235, and at
+// 64x64 tiles 16 frames of 300k Gaussians 1990 / 2030.  So from eight times what is
+// resident on, well above where the two meet.  Every pixel composites the same records
+// in the same order either way.  (Not in double or when pairs are counted, whose
+// kernels come with 256 threads alone.)
 bool narrow_parts(const Layout& L) {
   if (L.TW < 32 || L.real_size != 4 || L.count_pairs) return false;
   const int64_t parts = (int64_t)L.B * L.NT * (L.TW / 32) * (L.TH / 32);
-  return parts >= 8 * 152 * 3;
+  return parts >= 8 * kSMs * 3;
 }
 
 RenderGeom geom_of(const Layout& L) {

@@ -151,7 +151,7 @@ extern "C" gftorf_status gftorf_train_begin_shard(gftorf_train_state* state, flo
   if ((reinterpret_cast<uintptr_t>(state) & 7) != 0) return GFTORF_ERR_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   launch(train_begin_kernel, 1, 256, 0, st, state, n_bg ? bg : nullptr, (int)n_bg, seed,
-                                        (uint64_t)bg_offset, (uint64_t)bg_stride);
+         (uint64_t)bg_offset, (uint64_t)bg_stride);
   count_launches(1);
   return last_status();
 }
@@ -179,7 +179,7 @@ extern "C" gftorf_status gftorf_l2_loss_scaled(const gftorf_dims* dims, const fl
                    (reinterpret_cast<uintptr_t>(dL_dout) & 15) == 0;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   launch(l2_loss_kernel, sm_count() * 8, 256, 0, st, out, target, dL_dout, state, n_rows, L.C, FP,
-                                                 HW, (float)(2.0 / M), 1.0 / M, vec ? 1 : 0);
+         HW, (float)(2.0 / M), 1.0 / M, vec ? 1 : 0);
   count_launches(1);
   return last_status();
 }
