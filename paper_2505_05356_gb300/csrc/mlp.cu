@@ -949,16 +949,19 @@ __device__ __forceinline__ void encode_part(const float* __restrict__ means, con
 
 // warps 0-7: epilogue (warp w: TMEM lanes / rows 32 (w % 4) .. + 31, columns
 // 128 (w / 4) .. + 127); warp 8: TMA; warp 9: MMA.
-// What bounds the fused kernels is the 128 bytes a cycle that shared memory (and
+// The epilogue shares with the MMAs the 128 bytes a cycle that shared memory (and
 // the L1 data path behind every load) moves: for a tile's layer the MMAs read
 // 192 KB of operands (1536 cycles for 2048 of MMA), the weights arrive with 128 KB
 // and the epilogue stores 64 KB.  So the epilogue takes the accumulators as matrix
 // fragments (a lane: 16 columns of four rows), which needs a quarter of the bias
 // values per lane that one row of 64 columns did (those alone took 1024 cycles
 // per tile and layer, from global or shared memory alike), and stores them by
-// stmatrix.  300k rows of inference: 260 -> 191 us, 0.77 of the measured BF16
-// peak (timelines: 3300 -> 2300 cycles per tile and layer); training forward
-// 392 -> 319 us.  Sixteen epilogue warps measured the same.
+// stmatrix.  300k rows of inference: 260 -> 191 us (0.77 of the measured BF16
+// peak back to back, 0.73 by single calls), the tensor pipe active 51 -> 72 % of
+// the cycles; timelines: 3300 -> 2300 cycles per tile and layer.  Training forward
+// 392 -> 319 us, 33 -> 42 %: no unit is above 61 % there (L1 / shared memory 60,
+// DRAM 53), what is left is the chain of a tile's layers.  Sixteen epilogue warps
+// measured the same.
 constexpr int kFusedEpiWarps = 8;
 constexpr int kFusedEpiThreads = 32 * kFusedEpiWarps;
 constexpr int kFusedThreads = kFusedEpiThreads + 64;
