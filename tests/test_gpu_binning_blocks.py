@@ -69,6 +69,38 @@ def test_several_batches_per_chunk(W, H, tile, B, n):
     _compare(u, v, r, z, W, H, tile, tight=True)
 
 
+@pytest.mark.parametrize("W,H", [(640, 480), (1111, 777)])  # ranges by the scan, by their kernel
+def test_overflow_leaves_empty_ranges_and_the_next_binning_whole(W, H):
+    u, v, r, z = _case(5, 2, 3000, W, H, 20)
+    keys_o, vals_o, ranges_o = ora.bin_f32(u, v, r, z, W, H, 8, 8)
+    dev = [torch.as_tensor(a, device="cuda") for a in (u, v, r, z)]
+    lib, tiles = gftorf.load(), -(-W // 8) * -(-H // 8)
+    for cap, fits in ((len(vals_o) - 1, False), (len(vals_o), True)):
+        d = gftorf.Dims(3000, 2, W, H, 8, 8, 1, 1, gftorf.F32, 0, 0, 0, 0, max_instances=cap)
+        size = lib.gftorf_workspace_size(ctypes.byref(d))
+        ws = torch.empty(size + 256, dtype=torch.uint8, device="cuda")
+        at = ws.data_ptr() + (-ws.data_ptr()) % 256
+        vals = torch.empty(cap, dtype=torch.int32, device="cuda")
+        ranges = torch.empty((2 * tiles, 2), dtype=torch.int32, device="cuda")
+        count = torch.empty(1, dtype=torch.int64, device="cuda")
+        for _ in range(2):  # the second finds what the first left behind
+            assert lib.gftorf_sort_footprints(
+                ctypes.byref(d), *(t.data_ptr() for t in dev), None, vals.data_ptr(),
+                ranges.data_ptr(), count.data_ptr(), at, size,
+                torch.cuda.current_stream().cuda_stream) == gftorf.OK
+            n = ctypes.c_int64(0)
+            code = lib.gftorf_read_device_status(ctypes.byref(d), at, size, ctypes.byref(n),
+                                                 torch.cuda.current_stream().cuda_stream)
+            assert n.value == len(vals_o) == count.item()
+            assert code == (gftorf.OK if fits else gftorf.ERR_CAPACITY)
+            if fits:
+                np.testing.assert_array_equal(ranges.cpu().numpy().astype(np.uint32),
+                                              np.asarray(ranges_o, np.uint32).reshape(-1, 2))
+                np.testing.assert_array_equal(vals.cpu().numpy().astype(np.uint32), vals_o)
+            else:
+                assert not ranges.any().item()
+
+
 def _bin_us(W, H, tile, n):
     g = torch.Generator(device="cuda")
     g.manual_seed(n)
